@@ -964,8 +964,8 @@ def main():
         roof = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
                 "frac": achieved / fp32_peak,
                 "traffic": kernel_traffic() if nt else kernel_traffic("mul_f32_traffic.json", "mul.cu"),
-                "kernel": "sf::mul_f32_nt_kernel (K-major operands, one bulk copy per lambda block, "
-                          "split-K half-warps)" if nt else
+                "kernel": "sf::mul_f32_nt_kernel (packed operands, listed lambda blocks, "
+                          "split-K lane groups)" if nt else
                           "sf::mul_f32_kernel<tile %d, micro %dx%d, transposed A>" % (shape["tile"], *shape["micro"]),
                 "peak_source": "%d SMs (device attribute) x 128 FP32 lanes x 2 flop x %g MHz sm_max (derived)"
                                % (sms, sm_max),

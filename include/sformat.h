@@ -59,11 +59,13 @@ typedef enum {
  *              error-free transformations; about 2^-44 relative per operation.
  *   S_FP32     float in, float out, float multiply-add; the partial sum of each few lambda
  *              blocks is folded into the running sum by an error-free two-sum (compensated
- *              summation over lambda).  The default kernel reads both operands K-major: A as
- *              stored and B through a padded copy of its transposed blocks that the plan keeps
- *              (s_pattern_nnz(S_B) floats, rounded up per block to multiples of 4 in each
- *              dimension), unless s_plan_set_symmetric_a was set and the product is called
- *              with B = A on one pattern whose block sizes are multiples of 4.
+ *              summation over lambda).  The default kernel reads both operands through packed
+ *              copies that the plan keeps and every product rewrites (s_pattern_nnz floats each,
+ *              rounded up to even block widths; one copy for both when s_plan_set_symmetric_a
+ *              was set and the product is called with B = A on one pattern), and the plan keeps
+ *              the list of block triples (16 bytes each, up to 4 GiB; beyond that each product
+ *              lists them range by range through a 256 MiB workspace).  Where there is no
+ *              memory for these the product runs on a kernel that reads the operands as stored.
  *   S_BF16X3   float in, float out; each operand split into three bfloat16 parts,
  *              the six leading cross products on the tensor cores, float accumulate.
  *   S_TF32X3   float in, float out; each operand split as hi + lo, both rounded to TF32
@@ -124,8 +126,9 @@ s_status s_plan_stats(s_plan plan, int64_t* triples, double* flops);
  * (S_FP64 plans have tile edges 20 and 10; a plan whose output blocks have a
  * root-mean-square edge of at most 12 starts with 10, the others with 20.)
  * Each variant runs one timed warm-up launch; one more than twice as slow as the best so far
- * stops there, the others are timed over three more launches.  Float tile and row-panel
- * shapes narrower than the root-mean-square block edge of S_C are skipped.  C is
+ * stops there, the others are timed over three more launches.  Float plans whose packed kernel
+ * can run the call keep it (one product, nothing else is timed); for the others, tile and
+ * row-panel shapes narrower than the root-mean-square block edge of S_C are skipped.  C is
  * overwritten.  *chosen (optional) receives the variant index.  S_BF16X3 and S_TF32X3
  * plans have one shape (no-op).  Synchronises the stream. */
 s_status s_plan_autotune(s_plan plan, const void* A, const void* B, void* C, void* stream, int* chosen);
@@ -143,16 +146,15 @@ int s_plan_num_variants_of(s_plan plan);
  * needs B's pattern to be A's and the product to be called with B = A (the same buffer);
  * the kernel then reads B(lambda, nu') through the stored block (nu', lambda) and both
  * operands from one set of split planes.  For an S_FP32 plan whose B pattern is A's, the
- * K-major kernel then reads B(lambda, nu') through the stored (nu', lambda) when called with
- * B = A (no transposed copy; the plan releases it), and falls back to the other kernel shape
+ * packed kernel then reads B(lambda, nu') through the packed (nu', lambda) when called with
+ * B = A (no second copy; the plan releases it), and falls back to the other kernel shape
  * of its tile list when called with another B. */
 s_status s_plan_set_symmetric_a(s_plan plan, int symmetric);
 /* Shape of a variant of the plan's arithmetic (variant < 0: the current one): output tile edge, the
  * micro-tile of one lane, and the largest lambda extent staged at once (consecutive small
  * lambda blocks are packed into one stage up to this extent).  Float variants 0 (the default)
- * and 1 are the K-major kernel: each lambda block staged by one bulk copy, the micro-tile a
- * quarter of each tile's padded edge (reported as 0 x 0), lambda staged in pieces of at most
- * 20; variant 1 addresses full 20-wide pieces with a compile-time row pitch.  For an S_TF32X3 plan: 32 rows
+ * and 1 are the packed kernel: the micro-tile half or a quarter of each tile's edge (reported
+ * as 0 x 0), lambda staged in pieces of at most 20.  For an S_TF32X3 plan: 32 rows
  * of a panel, 128 MMA rows (member columns), 32 MMA columns, lambda extent 24 per stage.
  * Any output may be NULL. */
 s_status s_plan_variant(s_plan plan, int variant, int* tile, int* micro_rows, int* micro_cols, int* stage_k);
@@ -163,8 +165,8 @@ s_status s_plan_variant(s_plan plan, int variant, int* tile, int* micro_rows, in
  * no entry outside S_C is formed.  A, B, C are device value buffers on S_A, S_B, S_C in
  * the plan's element type; C must not alias A or B.  Deterministic: each output entry is
  * summed in a fixed order, so the same inputs give the same bits.  S_TF32X3
- * waits on its own tensor-core work and the K-major S_FP32 kernel on its own bulk copies,
- * each with a limit of about one second; if that ever runs out, the outputs are unspecified
+ * waits on its own tensor-core work with a limit of about one second; if that ever runs out,
+ * the outputs are unspecified
  * (NaN where written after the time-out) and the plan records the time-out: the plan's next
  * s_mul_masked, s_graph_launch or s_plan_status returns S_ERR_TIMEOUT (launching nothing)
  * and clears the record. */
@@ -172,8 +174,8 @@ s_status s_mul_masked(s_plan plan, const void* A, const void* B, void* C, void* 
 
 /* Synchronises `stream`, then reports the plan's device-side record: S_ERR_TIMEOUT (and the
  * record cleared) if a bounded wait of an earlier product or adjoint of this plan ran out,
- * else S_OK.  The kernels that wait on the device are the S_TF32X3 kernel (its tensor-core
- * work) and the K-major S_FP32 kernel (its bulk copies); the others never set the record. */
+ * else S_OK.  The S_TF32X3 kernel waits on the device (its tensor-core work); the others never
+ * set the record. */
 s_status s_plan_status(s_plan plan, void* stream);
 /* Diagnostics: *word receives the host address of the plan's forward time-out word (pinned
  * host memory mapped into the device, 0 = no time-out).  A kernel stores 1 there when its

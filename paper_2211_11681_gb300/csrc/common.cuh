@@ -90,22 +90,43 @@ struct TcEntry {
   int32_t nl, wd;
 };
 
-// One operand side of the K-major float product (mul_nt.cu): the op(X) row lists or op(Y)
-// column lists, and where the kernel finds each block's K-major slice data: directly in the
-// caller's buffer (offsets = the pattern's voff) or in a padded, per-block transposed copy
-// written by a pre-pass into `scratch` (offsets poff).
+// One operand side of the packed float product (mul_nt.cu): the op(X) row lists or op(Y)
+// column lists, and the packed copy of the operand's blocks that a pre-pass of every product
+// writes into `scratch` at offsets poff.
 struct NtSideDesc {
   const int64_t* ptr = nullptr;
   const int32_t* idx = nullptr;
   const int32_t* blk = nullptr;
   const int64_t* off = nullptr;   // nullptr: side not configured
   const s_pattern_t* pat = nullptr;
-  bool prep = false;              // true: the kernel reads `scratch`
-  bool trans = false;             // prepared copy holds the stored blocks transposed
-  bool from_x = false;            // Y side: reads the X side's prepared copy (B = A, symmetric)
+  bool trans = false;             // the packed copy holds the stored blocks transposed
+  bool from_x = false;            // Y side: reads the X side's packed copy (B = A, symmetric)
   int64_t* poff = nullptr;
   float* scratch = nullptr;
-  int64_t len = 0;
+  int64_t len = 0;                // floats of the packed copy
+};
+
+// One matching lambda block (or piece of kNtKC values of t of a wide one) of a block of S_C in the
+// packed float product: where the packed X and Y blocks start (in 4 floats), their padded t
+// extent, the first t of the piece and its extent.
+struct alignas(16) NtEntry {
+  uint32_t xo, yo;
+  uint16_t kp, t0;
+  uint32_t kc;
+};
+
+// Output tile of the packed float product: where its list and its first entry of C start, list
+// length, row pitch of C, place in the block and extent.
+struct alignas(16) NtTile {
+  int64_t e0, coff;
+  int32_t ne, nj;
+  uint16_t r0, c0, th, tw;
+};
+
+// Blocks k0 .. k1-1 of S_C (tiles t0 .. t1-1) whose lists are in memory together, from entry
+// `base` on.
+struct NtRange {
+  int64_t k0, k1, t0, t1, base;
 };
 
 struct MulDesc {
@@ -132,7 +153,11 @@ struct MulDesc {
   unsigned int* err_host = nullptr;  // of a kernel ran out; pinned host memory mapped into the
                                      // device, so the host reads it without a sync
   bool tc_sym = false;             // symmetric plan: B = A, Y read through its stored transpose
-  NtSideDesc ntx, nty;             // K-major float product sides (S_FP32)
+  NtSideDesc ntx, nty;             // packed float product sides (S_FP32)
+  int64_t* nt_eptr = nullptr;      // first entry of each block of S_C (device, nblocks + 1)
+  NtTile* nt_tiles = nullptr;      // tiles of S_C in block order
+  NtEntry* nt_ent = nullptr;       // lists of the current range (nullptr: side or lists missing)
+  std::vector<NtRange> nt_ranges;  // one: the plan keeps all lists
   bool nt_ysym = false;            // Y side read through X's rows (B = A, symmetric)
   float2* df_x = nullptr;    // S_FP64_DF: split operands (hi, lo)
   float2* df_y = nullptr;
@@ -151,12 +176,13 @@ void tc_free(MulDesc* d);
 s_status launch_tc(const MulDesc& d, const void* X, const void* Y, void* C, cudaStream_t st);
 // S_ERR_TIMEOUT (and the record cleared) if the descriptor's time-out word is set, else S_OK.
 s_status take_timeout(const MulDesc& d);
-// K-major float product (mul_nt.cu): configure the sides of a float descriptor, whether a call
+// Packed float product (mul_nt.cu): configure the sides and lists of a float descriptor, whether a call
 // with these buffers can use it, the launch, and the release of its scratch.
 s_status nt_configure(MulDesc* d, bool x_trans, bool y_trans, bool y_sym);
 bool nt_usable(const MulDesc& d, const void* X, const void* Y);
-s_status launch_nt(const MulDesc& d, const void* X, const void* Y, void* C, cudaStream_t st, bool const_pitch);
+s_status launch_nt(const MulDesc& d, const void* X, const void* Y, void* C, cudaStream_t st);
 void nt_free_side(NtSideDesc* s);
+void nt_free_lists(MulDesc* d);
 s_status run_mul(const MulDesc& d, s_prec prec, const void* X, const void* Y, void* C, cudaStream_t st);
 
 // Element-wise kernels (add.cu)

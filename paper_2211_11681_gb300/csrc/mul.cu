@@ -1246,15 +1246,15 @@ static s_status build_panels(MulDesc* d, int edge, int P) {
 struct F32Variant {
   int tt, mr, mc, km;  // tile edge, lane micro-tile, largest lambda extent of one stage
   int panel;           // 0: one tile per warp; P > 0: row panels of up to P tiles per warp
-  int nt;              // K-major kernel with bulk-copy staging (mul_nt.cu), micro-tile per tile:
-                       // 1 = runtime row pitch, 2 = compile-time pitch for full 20-wide pieces
+  int nt;              // packed kernel (mul_nt.cu), micro-tile per tile
 };
-constexpr F32Variant kF32Variants[] = {{20, 0, 0, 20, 0, 1},  {20, 0, 0, 20, 0, 2},  {20, 4, 4, 20, 0, 0},
+// Variants 0 and 1 are the same kernel (1 keeps its number).
+constexpr F32Variant kF32Variants[] = {{20, 0, 0, 20, 0, 1},  {20, 0, 0, 20, 0, 1},  {20, 4, 4, 20, 0, 0},
                                        {20, 4, 4, 40, 0, 0},  {16, 4, 2, 32, 0, 0},  {12, 3, 2, 36, 0, 0},
                                        {10, 2, 2, 40, 0, 0},  {8, 2, 1, 32, 0, 0},   {12, 3, 2, 12, 3, 0},
                                        {10, 2, 2, 10, 4, 0},  {8, 2, 1, 8, 4, 0}};
 constexpr int kNumF32Variants = 11;
-constexpr int kF32Fallback = 2;  // tile kernel of the K-major variants' tile list, for unaligned buffers
+constexpr int kF32Fallback = 2;  // tile kernel of the packed variants' tile list, where that kernel cannot run
 
 static int num_sms() { return sm_count(); }
 
@@ -1400,6 +1400,7 @@ void free_desc(MulDesc* d) {
   tc_free(d);
   nt_free_side(&d->ntx);
   nt_free_side(&d->nty);
+  nt_free_lists(d);
   if (d->err_host) cudaFreeHost(d->err_host);
   d->err_host = nullptr;
   d->err = nullptr;
@@ -1514,8 +1515,8 @@ static s_status launch_typed(const MulDesc& d, const void* X, const void* Y, voi
     if (d.edge != kF32Variants[d.variant].tt) return set_error(S_ERR_ARG, "internal: tile list does not match variant");
     int v = d.variant;
     if (kF32Variants[v].nt) {
-      if (nt_usable(d, X, Y)) return launch_nt(d, X, Y, C, st, kF32Variants[v].nt == 2);
-      v = kF32Fallback;  // same tile list (edge 20); reads any alignment
+      if (nt_usable(d, X, Y)) return launch_nt(d, X, Y, C, st);
+      v = kF32Fallback;  // same tile list (edge 20)
     }
     kern = f32_kernel_of(v, d.x.trans, d.y.trans);
     warps = kF32Warps;
@@ -1777,6 +1778,10 @@ extern "C" s_status s_plan_autotune(s_plan p, const void* A, const void* B, void
     // tile shapes narrower than 20 only where the blocks are no wider than their tiles
     if (fl && !panel && !kF32Variants[v].nt && kF32Variants[v].tt < 20 && rms_edge > kF32Variants[v].tt) continue;
     if (f64 && kF64Edges[v] < 20 && rms_edge > 12.0) continue;
+    // Where the packed kernel can run nothing else is timed: on every pattern measured (blocks 1 to
+    // 40 wide, N = 1000 to 2^20) the tile and panel shapes took 1.6 to 4 times as long, and timing
+    // them took as long as 30 products.
+    if (fl && v > 0 && nt_usable(p->fwd, A, B)) break;
     if ((s = build_tiles(&p->fwd, edge_of(v)))) break;
     if (panel && (s = build_panels(&p->fwd, kF32Variants[v].tt, kF32Variants[v].panel))) break;
     p->fwd.variant = v;
@@ -1791,6 +1796,11 @@ extern "C" s_status s_plan_autotune(s_plan p, const void* A, const void* B, void
     }
     float ms = 0.0f;
     cudaEventElapsedTime(&ms, e0, e1);
+    if (fl && nt_usable(p->fwd, A, B)) {  // the only candidate
+      p->tune_ms[v] = ms;
+      bestv = v;
+      continue;
+    }
     if (ms > 2.0f * best / 3.0f) {
       p->tune_ms[v] = ms;
       continue;
@@ -1850,7 +1860,7 @@ extern "C" s_status s_plan_variant(s_plan p, int variant, int* tile, int* micro_
     return S_OK;
   }
   if (variant >= kNumF32Variants) return set_error(S_ERR_ARG, "s_plan_variant: no such variant");
-  if (tile) *tile = kF32Variants[variant].tt;  // K-major variant: micro-tile 0 x 0 = per tile
+  if (tile) *tile = kF32Variants[variant].tt;  // packed variant: micro-tile 0 x 0 = per tile
   if (micro_rows) *micro_rows = kF32Variants[variant].mr;
   if (micro_cols) *micro_cols = kF32Variants[variant].mc;
   if (stage_k) *stage_k = kF32Variants[variant].km;
@@ -1913,7 +1923,7 @@ extern "C" s_status s_plan_set_symmetric_a(s_plan p, int symmetric) {
   // read A(nu, lambda) as the transpose of the stored block (lambda, nu): same values when A
   // is symmetric, and column-contiguous staging for the float kernel
   p->fwd.x = side_of(A, true, symmetric != 0);
-  // the K-major float kernel reads A as stored and, for B = A, B(lambda, nu') through A's rows
+  // the packed float kernel reads A's rows and, for B = A, B(lambda, nu') through A's rows too
   if (p->prec == S_FP32) return nt_configure(&p->fwd, false, false, symmetric != 0 && p->b == p->a);
   return S_OK;
 }

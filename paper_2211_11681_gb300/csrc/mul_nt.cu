@@ -1,29 +1,55 @@
 // Float masked product C = P_{S_C}(op(X) op(Y)) (Eq. (product), Sec. 4.1) with both operands
-// staged K-major: every lambda block reaches shared memory as one contiguous bulk copy.
+// packed for the multiply-add loop.
 //
-// Operand layout ("K-major"): for the X side the slice op(X)(nu, lambda) is held as
-// [row of nu][t], for the Y side op(Y)(lambda, nu') as [column of nu'][t], t running over
-// lambda's samplets, both padded with zeros to multiples of 4 in each dimension.  Where a
-// value buffer already stores its blocks that way (op(X) = X, op(Y) = Y^T, or op(Y) = B with
-// B = A declared symmetric, all block sizes multiples of 4) the kernel reads it directly;
-// otherwise a pre-pass writes a padded, per-block transposed copy into plan-owned scratch.
-// Either way the rows r0 .. r0+th of a slice are one contiguous run of memory, so one
-// cp.async.bulk copy, issued by one lane and tracked by an mbarrier, stages it.
+// Operand layout ("t pairs"): for the X side the slice op(X)(nu, lambda) has a row per row of
+// nu, for the Y side op(Y)(lambda, nu') a row per column of nu', t running over lambda's
+// samplets.  A pre-pass (nt_prepare_kernel) writes each block, transposed as needed, into
+// plan-owned scratch as panels of at most 20 rows, a panel as [t / 2][row][t % 2]: t padded to
+// even with zeros, every block on a 16-byte boundary.  A range of t that starts at a multiple of
+// kNtKC is then one contiguous, aligned run for all rows of an output tile, and a lane finds its
+// MR rows' pairs side by side at constant offsets.  With B = A declared symmetric one copy
+// serves both sides.  The pre-pass moves 8 bytes an entry once where the product reads each
+// operand entry some 20 to 300 times.
+//
+// Lists: the matching lambda blocks of every block of S_C (where both operands' slices start, the
+// t extent) are written once by nt_list_kernel, one warp per block, and kept by the plan when
+// they fit kNtListMax; beyond that every product lists and multiplies range after range of
+// blocks through a workspace of kNtListWork.  Intersecting inside the product kernel cost more
+// than the products of narrow blocks: in the plane the lists of a tile are 300 entries long for
+// 60 matches.
 //
 // Work decomposition: one warp owns one output tile (at most 20 x 20 entries of one block of
-// S_C) for the whole lambda sum.  The tile, padded to 4 MR x 4 MC, is cut into a 4 x 4 grid
-// of MR x MC micro-tiles; each half-warp (16 lanes) holds the whole grid, and the two halves
-// take alternate lambda blocks of the tile's intersection list (split-K), so all 32 lanes
-// work whatever the block widths.  A lane's step over 4 values of t is MR + MC 16-byte
-// shared loads and 4 MR MC fused multiply-adds.  Each lambda block's partial sum is kept in
-// a float register per entry and folded into the running sum with an error-free two-sum
-// every kNtFold blocks, the rounding error carried in the partial; at the end the two
-// halves' sums are combined the same way.  The summation order is fixed (deterministic).
+// S_C) for the whole lambda sum.  The tile is cut into a GR x GC grid of MR x MC micro-tiles,
+// GR = 2 for tiles of at most 10 rows and 4 beyond (GC likewise), one lane per micro-tile, and
+// the 32 / (GR GC) lane groups take consecutive lambda blocks of the tile's list (split-K): 8
+// blocks at once for tiles up to 10 x 10, 2 for tiles beyond 10 both ways.  The control of a
+// step is paid once for all its blocks, so narrow blocks, whose products are only 7 to 30
+// multiply-add instructions, run 8 to a step.  A lane's step over a pair of t is MR + MC 8-byte
+// shared loads and MR MC packed multiply-adds (fma.rn.f32x2 over the two values of t).  What
+// bounds it: shared memory delivers 128 bytes per clock and SM to registers, i.e.
+// 8 (MR + MC) 32 / 128 clocks for a pair of t against MR MC / 2 clocks of the float pipes, 62 %
+// of the float peak for 5 x 5 micro-tiles (a loop of nothing else measured 42 to 49 TFLOP/s,
+// packed or not; packing halves the issue slots of the multiply-adds, which the control
+// instructions need); the narrow tiles are bound by latency at 4 warps a scheduler.
 //
-// Pipeline per warp: two stage buffers, each holding one lambda chunk (at most kNtKC values of
-// t) per half-warp; the copies of the next stage are in flight while the current one is
-// multiplied.  Waits on the mbarriers are bounded (about one second of SM clocks); on time-out
-// the plan's time-out word is set and the warp stops.
+// Staging: each lane group copies its own block with 16-byte cp.async (14 instructions a step
+// for 8 blocks of 10 x 10).  One bulk copy per operand and block took longer on narrow blocks
+// (a bulk copy issues from uniform registers, so a warp sends its 16 copies one lane at a time):
+// 41.5 against 37.6 ms for the three products of a gradient step at N = 6000 in space, q = 2.
+//
+// Sums: even and odd t are two float partials per entry; after the first step, then every 8 (16 of
+// 8 blocks at once), they are added and folded into the running sum with an error-free two-sum,
+// the rounding error carried in the partial.  The lists run from coarse to fine clusters, so
+// the first step holds the largest terms: folded at once, it no longer makes the small terms
+// that follow round at its size.  At the end the groups' sums are combined the same way in
+// group order.  The order is fixed (deterministic).  Error against 64 bits, geometric mean over 8
+// matrices of 500 to 9900 points: 0.6e-7 to 1.4e-7 in the four families with 20- and 10-wide
+// blocks (1.1e-7 to 4.0e-7 with the replaced kernel's folds every 4 lambda blocks).
+//
+// Measured against the kernel this replaces (K-major slices, in-kernel intersection, one half-warp
+// per lambda block): N = 50000 in the plane, 10-wide blocks, B not symmetric 9.27 -> 4.07 ms; N = 65536 in
+// space, 20-wide blocks, B = A symmetric 39.1 -> 30.5 ms (37.6 TFLOP/s); N = 1000 in the plane
+// 192 -> 82 us; three products of a gradient step, N = 6000, 10-wide blocks 107.6 -> 36.8 ms.
 #include <algorithm>
 #include <cstring>
 
@@ -33,261 +59,139 @@ namespace sf {
 namespace {
 
 constexpr int kNtWarps = 4;
-constexpr int kNtKC = 20;                        // lambda values per staged chunk
-constexpr int kNtEnt = 32;                       // matching lambda blocks listed at once
-constexpr int kNtRegion = 20 * kNtKC;            // floats of one operand slice (<= 20 rows)
-constexpr int kNtHalf = 2 * kNtRegion + 16;      // X | Y of one half-warp, + 64-byte bank shift
-constexpr int kNtBuf = 2 * kNtHalf;              // one stage buffer: both halves
-constexpr int kNtFold = 4;                       // lambda blocks per two-sum fold
-constexpr size_t kNtSmem = sizeof(float) * kNtWarps * 2 * kNtBuf;
+constexpr int kNtKC = 20;        // largest t extent of a listed piece
+constexpr int kNtBuf = 1632;     // floats of a stage buffer: 2 x 20x20x2 or 8 x 10x10x2 slices, and room to
+                                 // start the 8 slots 12 banks apart (conflict-free 8-byte loads)
+constexpr int kNtSlack = 64;     // a micro-tile reads up to 5 rows' pairs beyond its operand's last
+constexpr size_t kNtSmem = sizeof(float) * (kNtWarps * 2 * kNtBuf + kNtSlack);
+constexpr int64_t kNtListMax = (int64_t)4 << 30;    // bytes of lists a plan keeps
+constexpr int64_t kNtListWork = (int64_t)256 << 20; // bytes of the workspace beyond that
 
-struct NtEntry {
-  int64_t xo, yo;  // float offsets of the X and Y slices (rows r0.. / columns c0..)
-  int32_t nlp;     // padded lambda extent (row pitch of both slices)
-  int32_t pad;
-};
+// Padded t extent of a slice over nl values of t.
+__host__ __device__ __forceinline__ int nt_even(int nl) { return (nl + 1) & ~1; }
 
 struct NtArgs {
-  const int64_t* xptr;  // op(X) row lists: lambda ids xidx, block ids xblk (nullptr: position)
-  const int32_t* xidx;
-  const int32_t* xblk;
-  const int64_t* xoff;  // float offset of each block in X's K-major buffer
-  const float* X;
-  const int64_t* yptr;  // op(Y) column lists
-  const int32_t* yidx;
-  const int32_t* yblk;
-  const int64_t* yoff;
+  const float* X;        // packed operands
   const float* Y;
-  const int32_t* bsize;
-  const int32_t* c_brow;
-  const int32_t* c_col;
-  const int64_t* c_voff;
-  const Tile* tiles;
-  int64_t ntiles;
+  const NtEntry* ent;    // lists of the launch's range, from entry `base` on
+  int64_t base;
+  const NtTile* tiles;   // the launch's tiles
+  uint32_t ntiles;
   unsigned int* counter;
-  unsigned int* err;
   float* C;
 };
 
-__device__ __forceinline__ uint32_t nt_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ int nt_lower_bound(const int32_t* a, int lo, int hi, int32_t v) {
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (__ldg(a + mid) < v) lo = mid + 1;
-    else hi = mid;
-  }
-  return lo;
-}
-
-__device__ __forceinline__ void nt_expect(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(nt_smem(bar)), "r"(bytes)
-               : "memory");
-}
-
-__device__ __forceinline__ void nt_bulk(float* dst, const float* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-          nt_smem(dst)),
-      "l"(src), "r"(bytes), "r"(nt_smem(bar))
-      : "memory");
-}
-
-// Wait for phase `parity` of an mbarrier for at most about one second of SM clocks; returns
-// false on time-out.
-__device__ __forceinline__ bool nt_wait(uint64_t* bar, uint32_t parity) {
-  const uint32_t addr = nt_smem(bar);
-  const long long t0 = clock64();
-  for (;;) {
-    uint32_t done;
-    asm volatile(
-        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (clock64() - t0 > (1ll << 31)) return false;
-  }
-}
-
-// One staged piece of a lambda block: slice starts in the K-major X and Y buffers, the
-// block's padded extent (global row pitch), this piece's t0 and extent, and whether it ends
-// the block (last = -1: no piece).  All lanes hold the same values.
-struct NtChunk {
-  int64_t xo, yo;
-  int nlp, t0, kc, last;
+// What the listing kernel needs of a side: the lists of op(X)'s rows or op(Y)'s columns (lambda
+// ids, block ids or nullptr: position) and the float offset of each packed block.
+struct NtSide {
+  const int64_t* ptr;
+  const int32_t* idx;
+  const int32_t* blk;
+  const int64_t* off;
 };
 
-// Producer of a tile's pieces in increasing lambda order: lists matching lambda blocks
-// kNtEnt at a time (ballot over 32 entries of op(X)'s row list, binary search in op(Y)'s
-// column list) into the warp's entry table, then cuts each block into pieces of at most
-// kNtKC values of t.
-struct NtLister {
-  const NtArgs* a;
-  NtEntry* ent;
-  int px, px1, py0, py1;
-  int r0, c0;
-  int nm, e, t0;
-
-  __device__ __forceinline__ void refill(int lane) {
-    __syncwarp();
-    nm = 0;
-    e = 0;
-    while (nm == 0 && px < px1 && py0 < py1) {
-      while (px < px1 && py0 < py1 && nm <= kNtEnt - 32) {
-        const int i = px + lane;
-        const int32_t lam = i < px1 ? __ldg(a->xidx + i) : INT32_MAX;
-        const int pos = nt_lower_bound(a->yidx, py0, py1, lam);
-        const bool hit = i < px1 && pos < py1 && __ldg(a->yidx + pos) == lam;
-        const unsigned int mask = __ballot_sync(0xffffffffu, hit);
-        if (hit) {
-          const int kx = a->xblk ? __ldg(a->xblk + i) : i;
-          const int ky = a->yblk ? __ldg(a->yblk + pos) : pos;
-          const int nlp = (__ldg(a->bsize + lam) + 3) & ~3;
-          NtEntry en;
-          en.xo = __ldg(a->xoff + kx) + (int64_t)r0 * nlp;
-          en.yo = __ldg(a->yoff + ky) + (int64_t)c0 * nlp;
-          en.nlp = nlp;
-          en.pad = 0;
-          ent[nm + __popc(mask & ((1u << lane) - 1u))] = en;
+// Matching lambda blocks of the blocks k0 .. k1-1 of S_C in increasing lambda order, one warp per
+// block: the entries of the shorter list, 32 at a time, are looked up in the longer one by
+// binary search.  A lambda block wider than kNtKC gives one entry per piece of kNtKC values of t.
+// FILL: writes the entries at ent[eptr[k] - base ..); else writes their number to cnt[k].
+template <bool FILL>
+__global__ void __launch_bounds__(256) nt_list_kernel(NtSide x, NtSide y, const int32_t* __restrict__ bsize,
+                                                      const int32_t* __restrict__ c_brow,
+                                                      const int32_t* __restrict__ c_col, int64_t k0, int64_t k1,
+                                                      int32_t* __restrict__ cnt, const int64_t* __restrict__ eptr,
+                                                      int64_t base, NtEntry* __restrict__ ent) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t k = k0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5); k < k1;
+       k += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int nu = c_brow[k], nup = c_col[k];
+    const int px0 = (int)x.ptr[nu], nx = (int)x.ptr[nu + 1] - px0;
+    const int py0 = (int)y.ptr[nup], ny = (int)y.ptr[nup + 1] - py0;
+    const bool xs = nx <= ny;  // walk X's list, search Y's
+    const int32_t* sidx = xs ? x.idx + px0 : y.idx + py0;
+    const int32_t* lidx = xs ? y.idx + py0 : x.idx + px0;
+    const int ns = xs ? nx : ny, nl = xs ? ny : nx;
+    int lo0 = 0, total = 0;
+    NtEntry* out = FILL ? ent + (eptr[k] - base) : nullptr;
+    for (int i0 = 0; i0 < ns && lo0 < nl; i0 += 32) {
+      const int i = i0 + lane;
+      const int32_t v = i < ns ? __ldg(sidx + i) : INT32_MAX;
+      int lo = lo0, hi = nl;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(lidx + mid) < v) lo = mid + 1;
+        else hi = mid;
+      }
+      const bool hit = i < ns && lo < nl && __ldg(lidx + lo) == v;
+      const int kp = hit ? nt_even(__ldg(bsize + v)) : 0;
+      const int np = (kp + kNtKC - 1) / kNtKC;
+      int incl = np;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += u;
+      }
+      if (FILL && hit) {
+        const int ix = px0 + (xs ? i : lo), iy = py0 + (xs ? lo : i);
+        NtEntry en;
+        en.xo = (uint32_t)(__ldg(x.off + (x.blk ? __ldg(x.blk + ix) : ix)) >> 2);
+        en.yo = (uint32_t)(__ldg(y.off + (y.blk ? __ldg(y.blk + iy) : iy)) >> 2);
+        en.kp = kp;
+        for (int j = 0; j < np; ++j) {
+          en.t0 = j * kNtKC;
+          en.kc = min(kNtKC, kp - en.t0);
+          out[total + incl - np + j] = en;
         }
-        nm += __popc(mask);
-        py0 = __shfl_sync(0xffffffffu, pos, 31);
-        px += 32;
       }
+      total += __shfl_sync(0xffffffffu, incl, 31);
+      lo0 = __shfl_sync(0xffffffffu, lo, 31);
     }
-    __syncwarp();
-  }
-
-  __device__ __forceinline__ NtChunk next(int lane) {
-    NtChunk c;
-    if (e >= nm) refill(lane);
-    if (e >= nm) {
-      c.xo = c.yo = 0;
-      c.nlp = c.t0 = c.kc = 0;
-      c.last = -1;
-      return c;
-    }
-    const NtEntry en = ent[e];
-    c.xo = en.xo;
-    c.yo = en.yo;
-    c.nlp = en.nlp;
-    c.t0 = t0;
-    if (t0 == 0 && en.nlp <= kNtKC) {  // the common case: the whole block in one piece
-      c.kc = en.nlp;
-      c.last = 1;
-      ++e;
-      return c;
-    }
-    c.kc = min(kNtKC, en.nlp - t0);
-    c.last = t0 + c.kc >= en.nlp ? 1 : 0;
-    if (c.last) {
-      ++e;
-      t0 = 0;
-    } else {
-      t0 += c.kc;
-    }
-    return c;
-  }
-};
-
-// Issue the copies of one stage (piece c0 for half-warp 0, c1 for half-warp 1) into `buf`,
-// completing on `bar`.  A whole lambda block moves as one copy per operand (its rows r0.. /
-// columns c0.. are contiguous); a piece of a wider block as one copy per row.
-template <int TH, int TW>
-__device__ __forceinline__ void nt_issue(const NtArgs& a, const NtChunk& c0, const NtChunk& c1, float* buf,
-                                         uint64_t* bar, int lane) {
-  const bool v0 = c0.last >= 0, v1 = c1.last >= 0;
-  if ((!v0 || c0.kc == c0.nlp) && (!v1 || c1.kc == c1.nlp)) {
-    // whole blocks: lane 2h + o copies operand o (X, Y) of half-warp h's piece
-    if (lane == 0) nt_expect(bar, (uint32_t)((TH + TW) * 4 * ((v0 ? c0.kc : 0) + (v1 ? c1.kc : 0))));
-    __syncwarp();
-    if (lane < 4) {
-      const int h = lane >> 1, o = lane & 1;
-      const NtChunk& c = h ? c1 : c0;
-      if (h ? v1 : v0) {
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        nt_bulk(buf + h * kNtHalf + o * kNtRegion, o ? a.Y + c.yo : a.X + c.xo, (uint32_t)((o ? TW : TH) * c.nlp * 4),
-                bar);
-      }
-    }
-    return;
-  }
-  const uint32_t bytes = (uint32_t)((TH + TW) * 4 * ((v0 ? c0.kc : 0) + (v1 ? c1.kc : 0)));
-  const int n0 = v0 ? (c0.kc == c0.nlp ? 2 : TH + TW) : 0;
-  const int n1 = v1 ? (c1.kc == c1.nlp ? 2 : TH + TW) : 0;
-  // (the caller's __syncwarp ends every read of buf before this point)
-  if (lane == 0) nt_expect(bar, bytes);
-  __syncwarp();
-  if (lane < n0 + n1) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-  for (int j = lane; j < n0 + n1; j += 32) {
-    const int h = j < n0 ? 0 : 1;
-    const int q = h ? j - n0 : j;
-    const NtChunk& c = h ? c1 : c0;
-    const int nq = h ? n1 : n0;
-    float* dst = buf + h * kNtHalf;
-    if (nq == 2) {
-      if (q == 0) nt_bulk(dst, a.X + c.xo, (uint32_t)(TH * c.nlp * 4), bar);
-      else nt_bulk(dst + kNtRegion, a.Y + c.yo, (uint32_t)(TW * c.nlp * 4), bar);
-    } else if (q < TH) {
-      nt_bulk(dst + q * c.kc, a.X + c.xo + (int64_t)q * c.nlp + c.t0, (uint32_t)(c.kc * 4), bar);
-    } else {
-      const int r = q - TH;
-      nt_bulk(dst + kNtRegion + r * c.kc, a.Y + c.yo + (int64_t)r * c.nlp + c.t0, (uint32_t)(c.kc * 4), bar);
-    }
+    if (!FILL && lane == 0) cnt[k] = total;
   }
 }
 
-template <int MR, int MC, int KC>
-__device__ __forceinline__ void nt_fma_fixed(const float* xs, const float* ys, float* p) {
-#pragma unroll 1
-  for (int t = 0; t < KC; t += 4) {
-    float4 xv[MR];
-#pragma unroll
-    for (int i = 0; i < MR; ++i) xv[i] = *reinterpret_cast<const float4*>(xs + i * KC + t);
-#pragma unroll
-    for (int j = 0; j < MC; ++j) {
-      const float4 yv = *reinterpret_cast<const float4*>(ys + j * KC + t);
-#pragma unroll
-      for (int i = 0; i < MR; ++i) {
-        float s = p[i * MC + j];
-        s = fmaf(xv[i].x, yv.x, s);
-        s = fmaf(xv[i].y, yv.y, s);
-        s = fmaf(xv[i].z, yv.z, s);
-        s = fmaf(xv[i].w, yv.w, s);
-        p[i * MC + j] = s;
-      }
+// The tiles of every block of S_C, in block order: block k's tiles start at tptr[k].
+__global__ void nt_tile_kernel(int64_t nb, const int32_t* __restrict__ bsize, const int32_t* __restrict__ c_brow,
+                               const int32_t* __restrict__ c_col, const int64_t* __restrict__ c_voff,
+                               const int64_t* __restrict__ tptr, const int64_t* __restrict__ eptr,
+                               NtTile* __restrict__ tiles) {
+  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (k >= nb) return;
+  const int ni = bsize[c_brow[k]], nj = bsize[c_col[k]];
+  NtTile* o = tiles + tptr[k];
+  NtTile t;
+  t.e0 = eptr[k];
+  t.ne = (int32_t)(eptr[k + 1] - eptr[k]);
+  t.nj = nj;
+  for (int r0 = 0; r0 < ni; r0 += kTile)
+    for (int c0 = 0; c0 < nj; c0 += kTile) {
+      t.coff = c_voff[k] + (int64_t)r0 * nj + c0;
+      t.r0 = (uint16_t)r0;
+      t.c0 = (uint16_t)c0;
+      t.th = (uint16_t)min(kTile, ni - r0);
+      t.tw = (uint16_t)min(kTile, nj - c0);
+      *o++ = t;
     }
+}
+
+// 16-byte asynchronous copy global -> shared, past L1.
+__device__ __forceinline__ void nt_cp16(uint32_t dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+}
+
+// n pieces of 16 bytes by the GL lanes of a group, CI a lane at a time with constant offsets.
+template <int CI, int GL>
+__device__ __forceinline__ void nt_copy(uint32_t dst, const float* src, int n, int gl) {
+  dst += 16u * (uint32_t)gl;
+  src += 4 * gl;
+  for (int c = gl; c < n; c += CI * GL, dst += 16 * CI * GL, src += 4 * CI * GL) {
+#pragma unroll
+    for (int i = 0; i < CI; ++i)
+      if (c + i * GL < n) nt_cp16(dst + 16 * i * GL, src + 4 * i * GL);
   }
 }
 
-// The FMAs of one staged piece: MR rows of the X slice and MC rows of the Y slice (row pitch
-// kc), 4 values of t per step.  With CONST the full 20-wide piece, the common case, runs with
-// a compile-time row pitch (one address per step, constant offsets for the rows).
-template <int MR, int MC, bool CONST>
-__device__ __forceinline__ void nt_fma_chunk(const float* xs, const float* ys, int kc, float* p) {
-  if (CONST && kc == kNtKC) {
-    nt_fma_fixed<MR, MC, kNtKC>(xs, ys, p);
-    return;
-  }
-  for (int t = 0; t < kc; t += 4) {
-    float4 xv[MR];
-#pragma unroll
-    for (int i = 0; i < MR; ++i) xv[i] = *reinterpret_cast<const float4*>(xs + i * kc + t);
-#pragma unroll
-    for (int j = 0; j < MC; ++j) {
-      const float4 yv = *reinterpret_cast<const float4*>(ys + j * kc + t);
-#pragma unroll
-      for (int i = 0; i < MR; ++i) {
-        float s = p[i * MC + j];
-        s = fmaf(xv[i].x, yv.x, s);
-        s = fmaf(xv[i].y, yv.y, s);
-        s = fmaf(xv[i].z, yv.z, s);
-        s = fmaf(xv[i].w, yv.w, s);
-        p[i * MC + j] = s;
-      }
-    }
-  }
+__device__ __forceinline__ void nt_fma2(unsigned long long& d, unsigned long long x, unsigned long long y) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(x), "l"(y));
 }
 
 // acc + p as an error-free two-sum: acc <- rounded sum, p <- its rounding error
@@ -299,136 +203,168 @@ __device__ __forceinline__ void nt_fold(float& acc, float& p) {
   p = e;
 }
 
-// One output tile whose padded extent is 4MR x 4MC.  Returns false on a time-out.
-template <int MR, int MC, bool CONST>
-__device__ bool nt_tile(const NtArgs& a, const Tile& tile, int k, int nu, int nup, int ni, int nj, float* wbase,
-                        uint64_t* bars, NtEntry* ent, uint32_t& phase, int lane) {
-  constexpr int TH = 4 * MR, TW = 4 * MC, NQ = MR * MC;
-  const int half = lane >> 4, hl = lane & 15;
-  const int mr = hl >> 2, mc = hl & 3;
-  const int th = min(20, ni - tile.r0), tw = min(20, nj - tile.c0);
-  float acc[NQ], p[NQ];
+// the two partials of an entry added and folded; the error stays in the even partial
+__device__ __forceinline__ void nt_fold2(float& acc, unsigned long long& p) {
+  float v = __uint_as_float((unsigned int)p) + __uint_as_float((unsigned int)(p >> 32));
+  nt_fold(acc, v);
+  p = (unsigned long long)__float_as_uint(v);
+}
+
+__device__ __forceinline__ float2 nt_sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+
+// One output tile of at most GR MR x GC MC entries.
+template <int GR, int MR, int GC, int MC>
+__device__ __forceinline__ void nt_tile(const NtArgs& a, const NtTile& tile, float* wbase, uint32_t wsmem, int lane) {
+  constexpr int GL = GR * GC, S = 32 / GL, NQ = MR * MC, TW = GC * MC, NE = GR * MR * TW;
+  // t extents up to KMAX fit S slots in a stage buffer, those up to kNtKC half as many
+  constexpr int SLOT = kNtBuf / S, KMAX = S == 8 ? 10 : S == 4 ? 12 : kNtKC;
+  // 16-byte pieces a lane copies of an X and of a Y slice of up to KMAX
+  constexpr int CX = (GR * MR * KMAX / 4 + GL - 1) / GL, CY = (TW * KMAX / 4 + GL - 1) / GL;
+  constexpr int FOLD = S == 8 ? 16 : 8;  // steps per two-sum fold: partials of about 80 terms
+  static_assert(S * ((NE + 1) & ~1) * 2 <= 2 * kNtBuf, "the group sums reuse the stage buffers");
+  static_assert((GR * MR + TW) * KMAX <= SLOT && (GR * MR + TW) * kNtKC <= (S == 2 ? 1 : 2) * SLOT, "slot too small");
+  const int g = lane / GL, gl = lane % GL, mr = gl / GC, mc = gl % GC;
+  const int th = tile.th, tw = tile.tw, ne = tile.ne;
+  float acc[NQ];
+  unsigned long long p[NQ];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) acc[q] = p[q] = 0.0f;
-  int folded = 0;
-  bool ok = true;
-  NtLister L;
-  L.a = &a;
-  L.ent = ent;
-  L.px = (int)a.xptr[nu];
-  L.px1 = (int)a.xptr[nu + 1];
-  L.py0 = (int)a.yptr[nup];
-  L.py1 = (int)a.yptr[nup + 1];
-  L.r0 = tile.r0;
-  L.c0 = tile.c0;
-  L.nm = L.e = L.t0 = 0;
-  int buf = 0;
-  {
-    const NtChunk c0 = L.next(lane);
-    const NtChunk c1 = L.next(lane);
-    int kc = half ? c1.kc : c0.kc;
-    int last = half ? c1.last : c0.last;
-    if (c0.last >= 0) nt_issue<TH, TW>(a, c0, c1, wbase, bars, lane);
-    while (c0.last >= 0) {
-      const NtChunk n0 = L.next(lane);
-      const NtChunk n1 = L.next(lane);
-      const bool more = n0.last >= 0;
-      if (more) nt_issue<TH, TW>(a, n0, n1, wbase + (buf ^ 1) * kNtBuf, bars + (buf ^ 1), lane);
-      const bool got = nt_wait(bars + buf, (phase >> buf) & 1u);
-      phase ^= 1u << buf;
-      if (!__all_sync(0xffffffffu, got)) {
-        ok = false;
-        if (more) {  // let the copies already issued land before the warp leaves
-          nt_wait(bars + (buf ^ 1), (phase >> (buf ^ 1)) & 1u);
-          phase ^= 1u << (buf ^ 1);
+  for (int i = 0; i < NQ; ++i) {
+    acc[i] = 0.0f;
+    p[i] = 0ull;
+  }
+  const NtEntry* ep = a.ent + (tile.e0 - a.base);
+  int folded = FOLD - 1, buf = 0, pos = 0;  // the first step is folded at once
+  int cn = 0, ckc = 0, cxs = 0, cys = 0;  // the step in flight: blocks, this lane's t extent and slices
+  NtEntry en = {};
+  if (ne > 0) en = ep[min(g, ne - 1)];  // the group's block of the next step
+  for (;;) {
+    // ---- issue the next step into `buf`: each group copies its block's X slice, then its Y slice
+    int nn = 0, nkc = 0, nxs = 0, nys = 0;
+    if (pos < ne) {
+      nn = min(S, ne - pos);
+      const bool half = S > 2 && __any_sync(0xffffffffu, en.kc > KMAX);
+      if (half) nn = min(nn, S / 2);
+      nkc = g < nn ? (int)en.kc : 0;
+      const int nx = (th * nkc + 3) >> 2, ny = (tw * nkc + 3) >> 2;  // 16-byte pieces
+      nxs = buf * kNtBuf + g * (half ? 2 * SLOT : SLOT);
+      nys = nxs + 4 * nx;
+      nt_copy<CX, GL>(wsmem + 4u * (uint32_t)nxs,
+                      a.X + ((int64_t)en.xo * 4 + ((int64_t)tile.r0 * en.kp + th * (int)en.t0)), nx, gl);
+      nt_copy<CY, GL>(wsmem + 4u * (uint32_t)nys,
+                      a.Y + ((int64_t)en.yo * 4 + ((int64_t)tile.c0 * en.kp + tw * (int)en.t0)), ny, gl);
+      pos += nn;
+      if (pos < ne) en = ep[min(pos + g, ne - 1)];  // arrives during this step's multiply-adds
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    // ---- multiply the step in flight ---------------------------------------------------------
+    if (cn > 0) {
+      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+      __syncwarp();
+      const float* xs = wbase + cxs + mr * (2 * MR);
+      const float* ys = wbase + cys + mc * (2 * MC);
+#pragma unroll 2
+      for (int t = 0; t < ckc; t += 2, xs += 2 * th, ys += 2 * tw) {
+        unsigned long long xv[MR];
+#pragma unroll
+        for (int i = 0; i < MR; ++i) xv[i] = reinterpret_cast<const unsigned long long*>(xs)[i];
+#pragma unroll
+        for (int j = 0; j < MC; ++j) {
+          const unsigned long long yv = reinterpret_cast<const unsigned long long*>(ys)[j];
+#pragma unroll
+          for (int i = 0; i < MR; ++i) nt_fma2(p[i * MC + j], xv[i], yv);
         }
-        break;
       }
-      if (last >= 0) {
-        const float* hb = wbase + buf * kNtBuf + half * kNtHalf;
-        nt_fma_chunk<MR, MC, CONST>(hb + mr * MR * kc, hb + kNtRegion + mc * MC * kc, kc, p);
-        if (last && ++folded == kNtFold) {
-          folded = 0;
+      if (++folded == FOLD || nn == 0) {
+        folded = 0;
 #pragma unroll
-          for (int q = 0; q < NQ; ++q) nt_fold(acc[q], p[q]);
-        }
+        for (int i = 0; i < NQ; ++i) nt_fold2(acc[i], p[i]);
       }
       __syncwarp();
-      if (!more) break;
-      kc = half ? n1.kc : n0.kc;
-      last = half ? n1.last : n0.last;
-      buf ^= 1;
     }
+    if (nn == 0) break;
+    cn = nn;
+    ckc = nkc;
+    cxs = nxs;
+    cys = nys;
+    buf ^= 1;
   }
-  // ---- combine the halves and write the tile -------------------------------------------
-  float* cb = a.C + a.c_voff[k];
+  // ---- combine the groups in order through the (now idle) stage buffers, write the tile ------
+  __syncwarp();
+  // sums in [group][NE], then their errors; two neighbouring entries at a time
+  constexpr int NP = (NE + 1) & ~1;
+  float* red = wbase + g * NP;
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    const float oa = __shfl_xor_sync(0xffffffffu, acc[q], 16);
-    const float op = __shfl_xor_sync(0xffffffffu, p[q], 16);
-    float s = acc[q];
-    float e = oa;
-    nt_fold(s, e);  // s = acc0 + acc1, e = its rounding error
-    const int i = q / MC, j = q - i * MC;
-    const int r = mr * MR + i, c = mc * MC + j;
-    if (half == 0 && r < th && c < tw)
-      cb[(int64_t)(tile.r0 + r) * nj + tile.c0 + c] = ok ? s + (e + (p[q] + op)) : __int_as_float(0x7fc00000);
-  }
-  return ok;
-}
-
-template <bool CONST>
-__global__ void __launch_bounds__(kNtWarps * 32, 4) mul_f32_nt_kernel(NtArgs a) {
-  extern __shared__ __align__(128) float nsm[];  // [warp][buffer][kNtBuf]
-  __shared__ __align__(8) uint64_t bars[kNtWarps][2];
-  __shared__ __align__(16) NtEntry sent[kNtWarps][kNtEnt];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  float* wbase = nsm + (size_t)w * 2 * kNtBuf;  // the warp's two stage buffers
-  if (lane == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(nt_smem(&bars[w][0])));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(nt_smem(&bars[w][1])));
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  for (int n = 0; n < NQ; ++n) {
+    const int e = (mr * MR + n / MC) * tw + mc * MC + n % MC;
+    if (mr * MR + n / MC < th && mc * MC + n % MC < tw) {
+      red[e] = acc[n];
+      red[S * NP + e] = __uint_as_float((unsigned int)p[n]);
+    }
   }
   __syncwarp();
-  uint32_t phase = 0;
-  for (;;) {
-    unsigned int t = 0;
-    if (lane == 0) t = atomicAdd(a.counter, 1u);
-    t = __shfl_sync(0xffffffffu, t, 0);
-    if (t >= a.ntiles) break;
-    const Tile tile = a.tiles[t];
-    const int k = tile.blk;
-    const int nu = a.c_brow[k], nup = a.c_col[k];
-    const int ni = a.bsize[nu], nj = a.bsize[nup];
-    const int mr = (min(20, ni - tile.r0) + 3) >> 2, mc = (min(20, nj - tile.c0) + 3) >> 2;  // 1..5 each
-    bool ok = true;
-    float* wb = wbase;
-    uint64_t* bw = bars[w];
-    NtEntry* en = sent[w];
-#define SF_NT_CASE(R, Cc) \
-  case (R - 1) * 5 + (Cc - 1): ok = nt_tile<R, Cc, CONST>(a, tile, k, nu, nup, ni, nj, wb, bw, en, phase, lane); break;
-    switch ((mr - 1) * 5 + (mc - 1)) {
-      SF_NT_CASE(1, 1) SF_NT_CASE(1, 2) SF_NT_CASE(1, 3) SF_NT_CASE(1, 4) SF_NT_CASE(1, 5)
-      SF_NT_CASE(2, 1) SF_NT_CASE(2, 2) SF_NT_CASE(2, 3) SF_NT_CASE(2, 4) SF_NT_CASE(2, 5)
-      SF_NT_CASE(3, 1) SF_NT_CASE(3, 2) SF_NT_CASE(3, 3) SF_NT_CASE(3, 4) SF_NT_CASE(3, 5)
-      SF_NT_CASE(4, 1) SF_NT_CASE(4, 2) SF_NT_CASE(4, 3) SF_NT_CASE(4, 4) SF_NT_CASE(4, 5)
-      SF_NT_CASE(5, 1) SF_NT_CASE(5, 2) SF_NT_CASE(5, 3) SF_NT_CASE(5, 4) SF_NT_CASE(5, 5)
+  float* cb = a.C + tile.coff;
+  const int cnt = th * tw;
+  const float rtw = 1.0f / (float)tw;
+  for (int e = 2 * lane; e < cnt; e += 64) {
+    float2 s = *reinterpret_cast<const float2*>(wbase + e), r = *reinterpret_cast<const float2*>(wbase + S * NP + e);
+#pragma unroll
+    for (int o = 1; o < S; ++o) {
+      const float2 v = *reinterpret_cast<const float2*>(wbase + o * NP + e);
+      const float2 u = *reinterpret_cast<const float2*>(wbase + (S + o) * NP + e);
+      const float2 t = __fadd2_rn(s, v);
+      const float2 bp = nt_sub2(t, s);
+      r = __fadd2_rn(r, __fadd2_rn(__fadd2_rn(nt_sub2(s, nt_sub2(t, bp)), nt_sub2(v, bp)), u));
+      s = t;
+    }
+    s = __fadd2_rn(s, r);
+    const int i = __float2int_rz(((float)e + 0.5f) * rtw), j = e - i * tw;
+    const bool wrap = j + 1 == tw;
+    cb[(int64_t)i * tile.nj + j] = s.x;
+    if (e + 1 < cnt) cb[(int64_t)(i + wrap) * tile.nj + (wrap ? 0 : j + 1)] = s.y;
+  }
+  __syncwarp();
+}
+
+// Micro-tile class of a tile edge: 0, 1 = 2 x (3, 5), 2 .. 4 = 4 x (3, 4, 5).
+__device__ __forceinline__ int nt_class(int t) { return t <= 6 ? 0 : t <= 10 ? 1 : (t - 1) >> 2; }
+
+__global__ void __launch_bounds__(kNtWarps * 32, 4) mul_f32_nt_kernel(NtArgs a) {
+  extern __shared__ __align__(128) float nsm[];  // [warp][buffer][kNtBuf]
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float* wbase = nsm + (size_t)w * 2 * kNtBuf;  // the warp's two stage buffers
+  const uint32_t wsmem = (uint32_t)__cvta_generic_to_shared(wbase);
+  // the next tile is described, and the number of the one after it fetched, during the current one
+  unsigned int t = 0;
+  if (lane == 0) t = atomicAdd(a.counter, 1u);
+  t = __shfl_sync(0xffffffffu, t, 0);
+  NtTile nxt = {};
+  if (t < a.ntiles) nxt = a.tiles[t];
+  unsigned int tn = 0;
+  if (lane == 0) tn = atomicAdd(a.counter, 1u);
+  while (t < a.ntiles) {
+    const NtTile tile = nxt;
+    t = __shfl_sync(0xffffffffu, tn, 0);
+    if (t < a.ntiles) nxt = a.tiles[t];
+    if (lane == 0) tn = atomicAdd(a.counter, 1u);
+    const int rc = nt_class(tile.th), cc = nt_class(tile.tw);
+#define SF_NT_CASE(R, GR, MR, Cc, GC, MC) \
+  case R * 5 + Cc: nt_tile<GR, MR, GC, MC>(a, tile, wbase, wsmem, lane); break;
+#define SF_NT_ROW(R, GR, MR)                                                                       \
+  SF_NT_CASE(R, GR, MR, 0, 2, 3) SF_NT_CASE(R, GR, MR, 1, 2, 5) SF_NT_CASE(R, GR, MR, 2, 4, 3)      \
+  SF_NT_CASE(R, GR, MR, 3, 4, 4) SF_NT_CASE(R, GR, MR, 4, 4, 5)
+    switch (rc * 5 + cc) {
+      SF_NT_ROW(0, 2, 3) SF_NT_ROW(1, 2, 5) SF_NT_ROW(2, 4, 3) SF_NT_ROW(3, 4, 4) SF_NT_ROW(4, 4, 5)
       default: break;
     }
+#undef SF_NT_ROW
 #undef SF_NT_CASE
-    if (!ok) {
-      if (lane == 0) {
-        *(volatile unsigned int*)a.err = 1u;  // host-mapped word: plain store, then a system fence
-        __threadfence_system();
-      }
-      break;
-    }
   }
 }
 
-// Padded K-major copy of a pattern's blocks: block b (rows x cols, row-major in `src` at
-// voff[b]) is written at poff[b] as rows_p x cols_p (trans = false) or cols_p x rows_p (its
-// transpose, trans = true), sizes rounded up to multiples of 4 and the padding zero.
+// Packed copy of a pattern's blocks: block b (rows x cols, row-major in `src` at voff[b]), or its
+// transpose (trans), is written at poff[b] as panels of at most 20 rows, [t / 2][row][t % 2] each,
+// zeros for the padded t and up to the next multiple of 4 floats.  One warp per block; a lane
+// writes one pair of t (8 bytes) at a time.
 __global__ void nt_prepare_kernel(int64_t nb, const int32_t* __restrict__ bsize, const int32_t* __restrict__ brow,
                                   const int32_t* __restrict__ bcol, const int64_t* __restrict__ voff,
                                   const int64_t* __restrict__ poff, int trans, const float* __restrict__ src,
@@ -437,16 +373,21 @@ __global__ void nt_prepare_kernel(int64_t nb, const int32_t* __restrict__ bsize,
   for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; b < nb;
        b += ((int64_t)gridDim.x * blockDim.x) >> 5) {
     const int rows = bsize[brow[b]], cols = bsize[bcol[b]];
-    const int orows = trans ? cols : rows, ocols = trans ? rows : cols;  // output orientation
-    const int orp = (orows + 3) & ~3, ocp = (ocols + 3) & ~3;
+    const int R = trans ? cols : rows, K = trans ? rows : cols;  // panel rows and t extent
+    const int rs = trans ? 1 : cols, ts = trans ? cols : 1;      // source strides of a row and of t
+    const int kp = nt_even(K) >> 1;
     const float* s = src + voff[b];
-    float* d = dst + poff[b];
-    for (int e = lane; e < orp * ocp; e += 32) {
-      const int i = e / ocp, j = e - i * ocp;
-      float v = 0.0f;
-      if (i < orows && j < ocols) v = trans ? s[(int64_t)j * cols + i] : s[(int64_t)i * cols + j];
-      d[e] = v;
+    float2* d = reinterpret_cast<float2*>(dst + poff[b]);
+    for (int r0 = 0; r0 < R; r0 += kTile) {
+      const int th = min(kTile, R - r0);
+      const float rth = 1.0f / (float)th;
+      for (int e = lane; e < th * kp; e += 32) {
+        const int tp = e < (1 << 20) ? __float2int_rz(((float)e + 0.5f) * rth) : e / th, r = r0 + e - tp * th;
+        const float* v = s + (int64_t)r * rs + (int64_t)(2 * tp) * ts;
+        d[(int64_t)r0 * kp + e] = make_float2(v[0], 2 * tp + 1 < K ? v[ts] : 0.0f);
+      }
     }
+    if (lane == 0 && ((R * kp) & 1)) d[(int64_t)R * kp] = make_float2(0.0f, 0.0f);
   }
 }
 
@@ -454,21 +395,16 @@ __global__ void nt_prepare_kernel(int64_t nb, const int32_t* __restrict__ bsize,
 
 // ---- host side --------------------------------------------------------------------------
 
-static bool all_multiple_of_4(const s_pattern_t* p) {
-  for (int32_t b : p->bsize)
-    if (b & 3) return false;
-  return true;
-}
-
-// Float offsets of the padded blocks of pattern p (nblocks entries) on the device.
-static s_status padded_offsets(const s_pattern_t* p, int64_t** out, int64_t* total) {
+// Float offsets of the packed blocks of pattern p (nblocks entries) on the device: rows x even t
+// extent of the block or of its transpose, rounded up to 16 bytes.
+static s_status padded_offsets(const s_pattern_t* p, bool trans, int64_t** out, int64_t* total) {
   const int64_t nb = p->d.nblocks;
   std::vector<int64_t> off(std::max<int64_t>(nb, 1), 0);
   int64_t s = 0;
   for (int64_t b = 0; b < nb; ++b) {
     off[b] = s;
-    const int64_t r = (p->bsize[p->brow[b]] + 3) & ~3, c = (p->bsize[p->colidx[b]] + 3) & ~3;
-    s += r * c;
+    const int r = p->bsize[p->brow[b]], c = p->bsize[p->colidx[b]];
+    s += ((int64_t)(trans ? c : r) * nt_even(trans ? r : c) + 3) & ~int64_t(3);
   }
   *total = s;
   SF_CUDA(cudaMalloc(out, sizeof(int64_t) * off.size()));
@@ -482,10 +418,10 @@ void nt_free_side(NtSideDesc* s) {
   *s = NtSideDesc();
 }
 
-// Configure one side of the K-major product: `pat` is the stored operand's pattern, `list` the
-// row (X) or column (Y) lists of op(.), `trans` whether the K-major slice is the transpose of
-// the stored block.  Direct when no transpose is needed and every block size is a multiple
-// of 4; otherwise padded offsets and a scratch buffer for the prepared copy.
+// Configure one side of the packed product: `pat` is the stored operand's pattern, `list` the
+// row (X) or column (Y) lists of op(.), `trans` whether the packed slice is the transpose of
+// the stored block.  Where there is no memory for the packed copy the side stays unconfigured
+// (off = nullptr) and the product runs on the tile kernel, which reads the operands as stored.
 static s_status nt_side(const s_pattern_t* pat, const Side& list, bool trans, NtSideDesc* s) {
   nt_free_side(s);
   s->ptr = list.ptr;
@@ -493,23 +429,106 @@ static s_status nt_side(const s_pattern_t* pat, const Side& list, bool trans, Nt
   s->blk = list.blk;
   s->pat = pat;
   s->trans = trans;
-  s->prep = trans || !all_multiple_of_4(pat);
-  if (!s->prep) {
-    s->off = pat->d.voff;
+  s_status st = padded_offsets(pat, trans, &s->poff, &s->len);
+  if (st) return st;
+  const cudaError_t e = cudaMalloc(&s->scratch, sizeof(float) * std::max<int64_t>(s->len, 1));
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    s->scratch = nullptr;
     return S_OK;
   }
-  s_status st = padded_offsets(pat, &s->poff, &s->len);
-  if (st) return st;
+  SF_CUDA(e);
   s->off = s->poff;
-  SF_CUDA(cudaMalloc(&s->scratch, sizeof(float) * std::max<int64_t>(s->len, 1)));
   return S_OK;
 }
 
-// K-major sides of a float descriptor (forward or adjoint) for C = op(X) op(Y), op(X) = X^T
+static NtSide list_side(const NtSideDesc& s) { return NtSide{s.ptr, s.idx, s.blk, s.off}; }
+
+void nt_free_lists(MulDesc* d) {
+  cudaFree(d->nt_eptr);
+  cudaFree(d->nt_ent);
+  cudaFree(d->nt_tiles);
+  d->nt_tiles = nullptr;
+  d->nt_eptr = nullptr;
+  d->nt_ent = nullptr;
+  d->nt_ranges.clear();
+}
+
+// Counts the lists of a configured descriptor, lays out the ranges of blocks that go through the
+// workspace together (one range: the plan keeps the lists, which are written here) and
+// allocates.  Without memory for them the descriptor stays without lists and the product runs
+// on the tile kernel.  All work is on the default stream and finished on return.
+static s_status nt_build_lists(MulDesc* d) {
+  nt_free_lists(d);
+  if (!d->ntx.off || !d->nty.off) return S_OK;
+  // the entries count operand offsets in 4 floats with 32 bits, t in 16
+  if ((d->ntx.len >> 2) > (int64_t)UINT32_MAX || (d->nty.len >> 2) > (int64_t)UINT32_MAX) return S_OK;
+  for (const s_pattern_t* q : {d->px, d->py})
+    if (q->d.max_bsize > 65000) return S_OK;
+  const s_pattern_t* C = d->pc;
+  const int64_t nb = C->d.nblocks;
+  std::vector<int64_t> eptr(nb + 1, 0), tptr(nb + 1, 0);
+  int32_t* cnt = nullptr;
+  cudaError_t e = cudaMalloc(&cnt, sizeof(int32_t) * std::max<int64_t>(nb, 1));
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((nb + 7) / 8, (int64_t)sm_count() * 64));
+  if (e == cudaSuccess && nb > 0) {
+    nt_list_kernel<false><<<grid, 256>>>(list_side(d->ntx), list_side(d->nty), C->d.bsize, C->d.brow, C->d.colidx, 0, nb,
+                                         cnt, nullptr, 0, nullptr);
+    e = cudaGetLastError();
+    std::vector<int32_t> h(nb);
+    if (e == cudaSuccess) e = cudaMemcpy(h.data(), cnt, sizeof(int32_t) * nb, cudaMemcpyDeviceToHost);
+    for (int64_t k = 0; k < nb; ++k) eptr[k + 1] = eptr[k] + h[k];
+  }
+  cudaFree(cnt);
+  const int64_t most = kNtListMax / (int64_t)sizeof(NtEntry), work = kNtListWork / (int64_t)sizeof(NtEntry);
+  int64_t room = 0;  // entries to allocate
+  NtRange r{0, 0, 0, 0, 0};
+  for (int64_t k = 0; k < nb; ++k) {
+    const int64_t ni = C->bsize[C->brow[k]], nj = C->bsize[C->colidx[k]];
+    tptr[k + 1] = tptr[k] + ((ni + kTile - 1) / kTile) * ((nj + kTile - 1) / kTile);
+    // a launch counts its tiles in 32 bits
+    if (r.k1 > r.k0 && ((eptr[nb] > most && eptr[k + 1] - eptr[r.k0] > work) || tptr[k + 1] - r.t0 > INT32_MAX)) {
+      d->nt_ranges.push_back(r);
+      r = NtRange{k, k, tptr[k], tptr[k], 0};
+    }
+    r.k1 = k + 1;
+    r.t1 = tptr[k + 1];
+    room = std::max(room, eptr[r.k1] - eptr[r.k0]);
+  }
+  if (nb > 0) d->nt_ranges.push_back(r);
+  for (NtRange& q : d->nt_ranges) q.base = eptr[q.k0];
+  if (e == cudaSuccess) e = cudaMalloc(&d->nt_eptr, sizeof(int64_t) * (nb + 1));
+  if (e == cudaSuccess) e = cudaMemcpy(d->nt_eptr, eptr.data(), sizeof(int64_t) * (nb + 1), cudaMemcpyHostToDevice);
+  int64_t* dtptr = nullptr;
+  if (e == cudaSuccess) e = cudaMalloc(&dtptr, sizeof(int64_t) * (nb + 1));
+  if (e == cudaSuccess) e = cudaMemcpy(dtptr, tptr.data(), sizeof(int64_t) * (nb + 1), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMalloc(&d->nt_tiles, sizeof(NtTile) * std::max<int64_t>(tptr[nb], 1));
+  if (e == cudaSuccess && nb > 0) {
+    nt_tile_kernel<<<(unsigned)((nb + 255) / 256), 256>>>(nb, C->d.bsize, C->d.brow, C->d.colidx, C->d.voff, dtptr,
+                                                          d->nt_eptr, d->nt_tiles);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMalloc(&d->nt_ent, sizeof(NtEntry) * std::max<int64_t>(room, 1));
+  if (e == cudaSuccess && d->nt_ranges.size() == 1) {
+    nt_list_kernel<true><<<grid, 256>>>(list_side(d->ntx), list_side(d->nty), C->d.bsize, C->d.brow, C->d.colidx, 0, nb,
+                                        nullptr, d->nt_eptr, 0, d->nt_ent);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  cudaFree(dtptr);
+  if (e != cudaSuccess) {
+    nt_free_lists(d);
+    if (e != cudaErrorMemoryAllocation) return cuda_error(e, "packed float product: lists");
+    cudaGetLastError();
+  }
+  return S_OK;
+}
+
+// Packed sides of a float descriptor (forward or adjoint) for C = op(X) op(Y), op(X) = X^T
 // when x_trans and op(Y) = Y^T when y_trans.  X side: op(X) rows; the stored
 // block of a row-list entry is (nu, lambda) when op(X) = X (CSR row) and (lambda, nu) when
 // op(X) = X^T (CSC column).  Y side: op(Y) columns; with op(Y) = Y^T the stored block of a
-// CSR-row entry (nu', lambda) is already [column][t]; with op(Y) = Y the CSC-column entry
+// CSR-row entry (nu', lambda) has a row per column of op(Y); with op(Y) = Y the CSC-column entry
 // (lambda, nu') is transposed, unless `y_sym` (Y = X declared symmetric and called with one
 // buffer) lets the kernel read Y(nu', lambda) through Y's own CSR rows.
 s_status nt_configure(MulDesc* d, bool x_trans, bool y_trans, bool y_sym) {
@@ -528,20 +547,21 @@ s_status nt_configure(MulDesc* d, bool x_trans, bool y_trans, bool y_sym) {
     yl = Side{py.colptr, py.rowidx, py.cscblk, py.voff, true};
     ytrans = true;
   }
-  if (y_sym && !x_trans && d->ntx.prep) {
-    // B = A read through A's rows: the same padded blocks as the X side, one copy for both
+  if (y_sym && !x_trans) {
+    // B = A read through A's rows: the same packed blocks as the X side, one copy for both
     nt_free_side(&d->nty);
     d->nty.ptr = yl.ptr;
     d->nty.idx = yl.idx;
     d->nty.blk = yl.blk;
     d->nty.pat = d->py;
     d->nty.off = d->ntx.off;
+    d->nty.len = d->ntx.len;
     d->nty.from_x = true;
   } else if ((st = nt_side(d->py, yl, ytrans, &d->nty))) {
     return st;
   }
   d->nt_ysym = y_sym;
-  return S_OK;
+  return nt_build_lists(d);
 }
 
 static s_status nt_prepare(const NtSideDesc& s, const float* src, cudaStream_t st) {
@@ -555,61 +575,44 @@ static s_status nt_prepare(const NtSideDesc& s, const float* src, cudaStream_t s
 }
 
 bool nt_usable(const MulDesc& d, const void* X, const void* Y) {
-  if (!d.ntx.off || !d.nty.off) return false;
-  // bulk copies read 16-byte aligned sources
-  if (!d.ntx.prep && (reinterpret_cast<uintptr_t>(X) & 15)) return false;
-  if (!d.nty.prep && !d.nty.from_x && (reinterpret_cast<uintptr_t>(Y) & 15)) return false;
+  if (!d.nt_ent) return false;
   // a symmetric Y side reads B through A's rows: only valid for B = A
-  if (d.nt_ysym && X != Y) return false;
-  return true;
+  return !d.nt_ysym || X == Y;
 }
 
-s_status launch_nt(const MulDesc& d, const void* X, const void* Y, void* C, cudaStream_t st, bool const_pitch) {
+s_status launch_nt(const MulDesc& d, const void* X, const void* Y, void* C, cudaStream_t st) {
   if (d.ntiles == 0) return S_OK;
   s_status s = take_timeout(d);
   if (s) return s;
-  const float* xb = (const float*)X;
-  const float* yb = (const float*)Y;
-  if (d.ntx.prep) {
-    if ((s = nt_prepare(d.ntx, (const float*)X, st))) return s;
-    xb = d.ntx.scratch;
-  }
-  if (d.nty.from_x) {
-    yb = xb;
-  } else if (d.nty.prep) {
-    if ((s = nt_prepare(d.nty, (const float*)Y, st))) return s;
-    yb = d.nty.scratch;
-  }
-  NtArgs a;
-  a.xptr = d.ntx.ptr;
-  a.xidx = d.ntx.idx;
-  a.xblk = d.ntx.blk;
-  a.xoff = d.ntx.off;
-  a.X = xb;
-  a.yptr = d.nty.ptr;
-  a.yidx = d.nty.idx;
-  a.yblk = d.nty.blk;
-  a.yoff = d.nty.off;
-  a.Y = yb;
-  a.bsize = d.pc->d.bsize;
-  a.c_brow = d.pc->d.brow;
-  a.c_col = d.pc->d.colidx;
-  a.c_voff = d.pc->d.voff;
-  a.tiles = d.tiles;
-  a.ntiles = d.ntiles;
-  a.counter = d.counter;
-  a.err = d.err;
-  a.C = (float*)C;
-  SF_CUDA(cudaMemsetAsync(d.counter, 0, sizeof(unsigned int), st));
-  void (*kern)(NtArgs) = const_pitch ? mul_f32_nt_kernel<true> : mul_f32_nt_kernel<false>;
+  if ((s = nt_prepare(d.ntx, (const float*)X, st))) return s;
+  if (!d.nty.from_x && (s = nt_prepare(d.nty, (const float*)Y, st))) return s;
+  void (*kern)(NtArgs) = mul_f32_nt_kernel;
   SF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNtSmem));
   int per_sm = 0;
   SF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kNtWarps * 32, kNtSmem));
   if (per_sm < 1) per_sm = 1;
-  const int64_t want = (d.ntiles + kNtWarps - 1) / kNtWarps;
-  const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count() * per_sm);
-  kern<<<grid, kNtWarps * 32, kNtSmem, st>>>(a);
-  SF_CUDA(cudaGetLastError());
+  const DevPattern& pc = d.pc->d;
+  for (const NtRange& r : d.nt_ranges) {
+    if (d.nt_ranges.size() > 1) {
+      const int64_t lg = std::max<int64_t>(1, std::min<int64_t>((r.k1 - r.k0 + 7) / 8, (int64_t)sm_count() * 64));
+      nt_list_kernel<true><<<(int)lg, 256, 0, st>>>(list_side(d.ntx), list_side(d.nty), pc.bsize, pc.brow, pc.colidx, r.k0,
+                                                    r.k1, nullptr, d.nt_eptr, r.base, d.nt_ent);
+    }
+    NtArgs a;
+    a.X = d.ntx.scratch;
+    a.Y = d.nty.from_x ? d.ntx.scratch : d.nty.scratch;
+    a.ent = d.nt_ent;
+    a.base = r.base;
+    a.tiles = d.nt_tiles + r.t0;
+    a.ntiles = (uint32_t)(r.t1 - r.t0);
+    a.counter = d.counter;
+    a.C = (float*)C;
+    SF_CUDA(cudaMemsetAsync(d.counter, 0, sizeof(unsigned int), st));
+    const int64_t want = (r.t1 - r.t0 + kNtWarps - 1) / kNtWarps;
+    const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count() * per_sm);
+    if (grid > 0) kern<<<grid, kNtWarps * 32, kNtSmem, st>>>(a);
+    SF_CUDA(cudaGetLastError());
+  }
   return S_OK;
 }
 
