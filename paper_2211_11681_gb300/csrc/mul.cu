@@ -7,7 +7,9 @@
 // atomics).  The lambda set of a tile is the intersection of the sorted block-index lists
 // row(op(X), nu) and col(op(Y), nu'); a warp intersects them 32 entries of the X list at a
 // time by binary search in the Y list.  Warps take tiles from a device counter
-// (persistent grid sized to the SM count); tiles follow the block order of S_C.
+// (persistent grid sized to the SM count); tiles follow the block order of S_C.  The double
+// product deals several lambda blocks to the lanes of a warp (mul_f64_kernel); the default float
+// product lists its lambda blocks ahead (mul_nt.cu).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -103,22 +105,62 @@ __global__ void tile_fill_kernel(const int64_t* first, const int32_t* bsize, con
 }
 
 // ---- numeric kernels ----------------------------------------------------------------------
-constexpr int kWarps = 8;
-template <typename T>
-constexpr bool kCompensated = sizeof(T) == 4;
-// Double product: tile edge TT (20, or 10 for patterns of blocks at most about 10 wide),
-// every lane holding (TT^2 + 31) / 32 entries of the tile.
-template <typename T, int TT, bool TX, bool TY>
-__global__ void __launch_bounds__(kWarps * 32) mul_kernel(MulArgs a, const T* __restrict__ X,
-                                                          const T* __restrict__ Y, T* __restrict__ C) {
-  constexpr int kTile = TT;
-  constexpr int kPer = (TT * TT + 31) / 32;  // accumulators per lane
-  __shared__ T sX[kWarps][kTile * kTile];
-  __shared__ T sY[kWarps][kTile * kTile];
-  const int lane = threadIdx.x & 31;
-  const int w = threadIdx.x >> 5;
-  T* xs = sX[w];
-  T* ys = sY[w];
+// Double product.  One warp owns one output tile of at most 20 x 20 entries for the whole lambda
+// sum and takes S matching lambda blocks at a time (8 for tiles up to 10 x 10, 4 up to 200
+// entries, 2 beyond): the S blocks' slices are staged together, and the S th tw pairs of a
+// block and an entry are dealt to the lanes, kD64Slots accumulators each, so that all 32 lanes
+// hold work whatever the block widths; the S sums of an entry are added in order at the end.
+// What bounds it: the FP64 pipe, one warp instruction every 67 clocks a scheduler whether 1 or
+// 32 lanes are active (1.0 to 1.2 TFLOP/s measured with all 32), so an instruction's empty lanes
+// are the only cost that counts: one entry per lane and lambda block filled 78 % of the lanes
+// for 10 x 10 blocks and 56 % for 6 x 6, dealing 8 blocks fills 100 %.  Staging, listing and
+// addresses run in its shadow: 16 warps an SM, one stage buffer each, while one warp waits for
+// its copies the others multiply.
+// Whole blocks are staged as the runs they are stored as.  Measured against one entry per lane
+// and lambda block: N = 4096, 6- and 10-wide blocks 7.73 -> 5.99 ms; N = 20000, 9- and 10-wide blocks
+// 25.0 -> 20.0 ms (FP64 pipe 93 % active); N = 5000 in space, 20-wide blocks 62.4 -> 62.5 ms
+// (1.17 TFLOP/s, 96 % active, at the pipe either way).
+constexpr int kWarps = 4;
+constexpr int kD64Slots = 25;                 // accumulators of a lane: S th tw / 32 at most
+constexpr int kD64Buf = 1600;                 // doubles of a warp's stage buffer: S (th + tw) kc at most
+constexpr int kD64Ent = 48;                   // matching lambda blocks listed at once
+constexpr size_t kD64Smem = sizeof(double) * kWarps * kD64Buf;
+
+struct D64Entry {
+  int64_t xo, yo;  // entry offsets of op(X)'s and op(Y)'s blocks
+  int32_t nl;      // lambda's width
+  uint16_t t0, kc; // first t and t extent of this piece
+};
+
+// 8-byte asynchronous copy global -> shared.
+__device__ __forceinline__ void d64_cp(uint32_t dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
+}
+
+// rows x cols doubles at row pitch ld -> dst, packed.
+__device__ __forceinline__ void d64_stage(uint32_t dst, const double* src, int rows, int cols, int ld, int lane) {
+  const int len = rows * cols;
+  if (cols == ld) {
+#pragma unroll 4
+    for (int e = lane; e < len; e += 32) d64_cp(dst + 8u * (uint32_t)e, src + e);
+  } else {
+    const float rc = 1.0f / (float)cols;
+    for (int e = lane; e < len; e += 32) {
+      const int r = __float2int_rz(((float)e + 0.5f) * rc);
+      d64_cp(dst + 8u * (uint32_t)e, src + (int64_t)r * ld + (e - r * cols));
+    }
+  }
+}
+
+template <bool TX, bool TY>
+__global__ void __launch_bounds__(kWarps * 32, 4) mul_f64_kernel(MulArgs a, int edge, const double* __restrict__ X,
+                                                                 const double* __restrict__ Y, double* __restrict__ C) {
+  extern __shared__ __align__(16) double d64sm[];
+  __shared__ D64Entry sent[kWarps][kD64Ent];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double* base = d64sm + (size_t)w * kD64Buf;
+  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(base);
+  D64Entry* ent = sent[w];
   for (;;) {
     unsigned int t = 0;
     if (lane == 0) t = atomicAdd(a.counter, 1u);
@@ -128,83 +170,112 @@ __global__ void __launch_bounds__(kWarps * 32) mul_kernel(MulArgs a, const T* __
     const int k = tile.blk;
     const int nu = a.c_brow[k], nup = a.c_col[k];
     const int ni = a.bsize[nu], nj = a.bsize[nup];
-    const int th = min(kTile, ni - tile.r0), tw = min(kTile, nj - tile.c0);
-    const int nout = th * tw;
-    T acc[kPer], comp[kPer];
+    const int th = min(edge, ni - tile.r0), tw = min(edge, nj - tile.c0);
+    const int ne = th * tw;
+    // blocks to a step and the largest t extent staged: S (th + tw) KC <= kD64Buf and
+    // S ne <= 32 kD64Slots for every tile of at most 20 x 20
+    const int S = ne <= 100 && th + tw <= 20 ? 8 : ne <= 200 ? 4 : 2;
+    const int KC = S == 2 ? 20 : 10;
+    const int M = (S * ne + 31) >> 5;
+    double acc[kD64Slots];
+    int off[kD64Slots];  // slot m: block s of the step, entry (r, c): s << 16 | r << 8 | c
 #pragma unroll
-    for (int m = 0; m < kPer; ++m) acc[m] = comp[m] = T(0);
-    const int px0 = (int)a.x.ptr[nu], px1 = (int)a.x.ptr[nu + 1];
+    for (int m = 0; m < kD64Slots; ++m) {
+      acc[m] = 0.0;
+      const int i = min(lane + 32 * m, S * ne - 1);
+      const int s = i / ne, e = i - s * ne, r = e / tw;
+      off[m] = s << 16 | r << 8 | (e - r * tw);
+    }
+    const int px1 = (int)a.x.ptr[nu + 1];
+    int px = (int)a.x.ptr[nu];
     int py0 = (int)a.y.ptr[nup];
     const int py1 = (int)a.y.ptr[nup + 1];
-    for (int base = px0; base < px1 && py0 < py1; base += 32) {
-      const int i = base + lane;
-      const int32_t lam = i < px1 ? __ldg(a.x.idx + i) : INT32_MAX;
-      const int pos = lower_bound_dev(a.y.idx, py0, py1, lam);
-      const bool hit = i < px1 && pos < py1 && __ldg(a.y.idx + pos) == lam;
-      unsigned int mask = __ballot_sync(0xffffffffu, hit);
-      const int kx = hit ? (a.x.blk ? __ldg(a.x.blk + i) : i) : 0;
-      const int ky = hit ? (a.y.blk ? __ldg(a.y.blk + pos) : pos) : 0;
-      py0 = __shfl_sync(0xffffffffu, pos, 31);
-      while (mask) {
-        const int l = __ffs(mask) - 1;
-        mask &= mask - 1;
-        const int lm = __shfl_sync(0xffffffffu, lam, l);
-        const int bx = __shfl_sync(0xffffffffu, kx, l);
-        const int by = __shfl_sync(0xffffffffu, ky, l);
-        const int nl = a.bsize[lm];
-        const T* xb = X + a.x.voff[bx];
-        const T* yb = Y + a.y.voff[by];
-        for (int t0 = 0; t0 < nl; t0 += kTile) {
-          const int tk = min(kTile, nl - t0);
-          // op(X)(r0+r, t0+t) -> xs[r*tk+t];  op(Y)(t0+t, c0+c) -> ys[t*tw+c]
-          for (int e = lane; e < th * tk; e += 32) {
-            const int r = e / tk, tt = e - r * tk;
-            const int gr = tile.r0 + r, gt = t0 + tt;
-            xs[e] = TX ? xb[(int64_t)gt * ni + gr] : xb[(int64_t)gr * nl + gt];
+    int nm = 0, e0 = 0, piece = 0;  // entries listed, the next one, the window's next piece
+    for (;;) {
+      if (nm - e0 < S && px < px1 && py0 < py1) {
+        // list the next matching lambda blocks behind those left, wider ones in even pieces of at most KC
+        __syncwarp();
+        const D64Entry left = ent[min(e0 + lane, kD64Ent - 1)];
+        __syncwarp();
+        nm -= e0;
+        e0 = 0;
+        if (lane < nm) ent[lane] = left;
+        while (px < px1 && py0 < py1 && nm <= kD64Ent - 32) {
+          const int i = px + lane;
+          const int32_t lam = i < px1 ? __ldg(a.x.idx + i) : INT32_MAX;
+          const int pos = lower_bound_dev(a.y.idx, py0, py1, lam);
+          const bool hit = i < px1 && pos < py1 && __ldg(a.y.idx + pos) == lam;
+          const int nl = hit ? a.bsize[lam] : 0;
+          const int np = (nl + KC - 1) / KC;
+          const unsigned int mask = __ballot_sync(0xffffffffu, piece < np);
+          if (piece < np) {
+            const int kx = a.x.blk ? __ldg(a.x.blk + i) : i;
+            const int ky = a.y.blk ? __ldg(a.y.blk + pos) : pos;
+            const int len = (nl + np - 1) / np, t0 = piece * len;
+            ent[nm + __popc(mask & ((1u << lane) - 1u))] =
+                D64Entry{a.x.voff[kx], a.y.voff[ky], nl, (uint16_t)t0, (uint16_t)min(len, nl - t0)};
           }
-          for (int e = lane; e < tk * tw; e += 32) {
-            const int tt = e / tw, c = e - tt * tw;
-            const int gt = t0 + tt, gc = tile.c0 + c;
-            ys[e] = TY ? yb[(int64_t)gc * nl + gt] : yb[(int64_t)gt * nj + gc];
+          nm += __popc(mask);
+          if (__any_sync(0xffffffffu, piece + 1 < np)) {
+            ++piece;
+            continue;
           }
-          __syncwarp();
-#pragma unroll
-          for (int m = 0; m < kPer; ++m) {
-            const int e = lane + 32 * m;
-            if (e < nout) {
-              const int r = e / tw, c = e - r * tw;
-              const T* xr = xs + r * tk;
-              const T* yc = ys + c;
-              if (kCompensated<T>) {
-                // float: partial over this lambda block, then an error-free two-sum into
-                // (acc, comp); the long lambda-sums would otherwise lose ~1e-6 (Sec. 4.1
-                // sums over all lambda levels)
-                T s = T(0);
-                for (int tt = 0; tt < tk; ++tt) s = fma(xr[tt], yc[tt * tw], s);
-                const T hi = acc[m] + s;
-                const T bp = hi - acc[m];
-                comp[m] += (acc[m] - (hi - bp)) + (s - bp);
-                acc[m] = hi;
-              } else {
-                T s = acc[m];
-                for (int tt = 0; tt < tk; ++tt) s = fma(xr[tt], yc[tt * tw], s);
-                acc[m] = s;
-              }
-            }
-          }
-          __syncwarp();
+          piece = 0;
+          py0 = __shfl_sync(0xffffffffu, pos, 31);
+          px += 32;
         }
+        __syncwarp();
       }
-    }
-    T* cb = C + a.c_voff[k];
+      const int n = min(S, nm - e0);
+      if (n <= 0) break;
+      int kc = 0;
+      for (int s = 0; s < n; ++s) kc = max(kc, (int)ent[e0 + s].kc);
+      // stage in the order the blocks are stored: X as [r][tt] (TX: [tt][r]), Y as [tt][c] (TY:
+      // [c][tt]), so that whole blocks are one run
+      const int sx = th * kc, ss = sx + kc * tw;
+      for (int s = 0; s < n; ++s) {
+        const D64Entry en = ent[e0 + s];
+        const int nl = en.nl, tb = en.t0, kw = en.kc;
+        const double* xb = X + en.xo + (TX ? (int64_t)tb * ni + tile.r0 : (int64_t)tile.r0 * nl + tb);
+        const double* yb = Y + en.yo + (TY ? (int64_t)tile.c0 * nl + tb : (int64_t)tb * nj + tile.c0);
+        const uint32_t dx = sbase + 8u * (uint32_t)(s * ss), dy = dx + 8u * (uint32_t)sx;
+        d64_stage(dx, xb, TX ? kw : th, TX ? th : kw, TX ? ni : nl, lane);
+        d64_stage(dy, yb, TY ? tw : kw, TY ? kw : tw, TY ? nl : nj, lane);
+      }
+      asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+      __syncwarp();
+      // slots of the step's blocks; a slot runs to the largest t extent of its lanes' blocks
 #pragma unroll
-    for (int m = 0; m < kPer; ++m) {
-      const int e = lane + 32 * m;
-      if (e < nout) {
-        const int r = e / tw, c = e - r * tw;
-        cb[(int64_t)(tile.r0 + r) * nj + tile.c0 + c] = kCompensated<T> ? acc[m] + comp[m] : acc[m];
+      for (int m = 0; m < kD64Slots; ++m) {
+        if (32 * m >= n * ne) break;
+        const int o = off[m], s = o >> 16;
+        const int kl = s < n ? (int)ent[e0 + s].kc : 0;
+        const int ku = __reduce_max_sync(0xffffffffu, kl);
+        const int r = (o >> 8) & 255, c = o & 255;
+        const double* xp = base + s * ss + (TX ? r : r * kl);
+        const double* yp = base + s * ss + sx + (TY ? c * kl : c);
+        double v = acc[m];
+#pragma unroll 2
+        for (int tt = 0; tt < ku; ++tt, xp += TX ? th : 1, yp += TY ? 1 : tw)
+          if (tt < kl) v = fma(*xp, *yp, v);
+        acc[m] = v;
       }
+      __syncwarp();
+      e0 += n;
     }
+    // the S sums of an entry, added in order
+#pragma unroll
+    for (int m = 0; m < kD64Slots; ++m)
+      if (lane + 32 * m < S * ne) base[lane + 32 * m] = acc[m];
+    __syncwarp();
+    double* cb = C + a.c_voff[k] + (int64_t)tile.r0 * nj + tile.c0;
+    for (int e = lane; e < ne; e += 32) {
+      double v = base[e];
+      for (int s = 1; s < S; ++s) v += base[s * ne + e];
+      const int r = e / tw, c = e - r * tw;
+      cb[(int64_t)r * nj + c] = v;
+    }
+    __syncwarp();
   }
 }
 
@@ -1491,8 +1562,7 @@ static s_status launch_f32_panel(const MulDesc& d, const void* X, const void* Y,
   return S_OK;
 }
 
-template <typename T>
-static s_status launch_typed(const MulDesc& d, const void* X, const void* Y, void* C, cudaStream_t st) {
+static MulArgs mul_args(const MulDesc& d) {
   MulArgs a;
   a.x = dev_side(d.x);
   a.y = dev_side(d.y);
@@ -1503,41 +1573,47 @@ static s_status launch_typed(const MulDesc& d, const void* X, const void* Y, voi
   a.tiles = d.tiles;
   a.ntiles = d.ntiles;
   a.counter = d.counter;
+  return a;
+}
+
+static s_status launch_f32(const MulDesc& d, const void* X, const void* Y, void* C, cudaStream_t st) {
   if (d.ntiles == 0) return S_OK;
-  SF_CUDA(cudaMemsetAsync(d.counter, 0, sizeof(unsigned int), st));
-  int per_sm = 0;
-  using K = void (*)(MulArgs, const T*, const T*, T*);
-  K kern;
-  int warps;
-  size_t dsmem = 0;
-  if constexpr (sizeof(T) == 4) {
-    if (kF32Variants[d.variant].panel) return launch_f32_panel(d, X, Y, C, st);
-    if (d.edge != kF32Variants[d.variant].tt) return set_error(S_ERR_ARG, "internal: tile list does not match variant");
-    int v = d.variant;
-    if (kF32Variants[v].nt) {
-      if (nt_usable(d, X, Y)) return launch_nt(d, X, Y, C, st);
-      v = kF32Fallback;  // same tile list (edge 20)
-    }
-    kern = f32_kernel_of(v, d.x.trans, d.y.trans);
-    warps = kF32Warps;
-    dsmem = f32_smem(v);
-    SF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsmem));
-  } else {
-    const int tt = kF64Edges[d.variant < kNumF64Variants ? d.variant : 0];
-    if (d.edge != tt) return set_error(S_ERR_ARG, "internal: tile list does not match the double variant");
-    if (tt == 10)
-      kern = d.x.trans ? (d.y.trans ? mul_kernel<T, 10, true, true> : mul_kernel<T, 10, true, false>)
-                       : (d.y.trans ? mul_kernel<T, 10, false, true> : mul_kernel<T, 10, false, false>);
-    else
-      kern = d.x.trans ? (d.y.trans ? mul_kernel<T, 20, true, true> : mul_kernel<T, 20, true, false>)
-                       : (d.y.trans ? mul_kernel<T, 20, false, true> : mul_kernel<T, 20, false, false>);
-    warps = kWarps;
+  if (kF32Variants[d.variant].panel) return launch_f32_panel(d, X, Y, C, st);
+  if (d.edge != kF32Variants[d.variant].tt) return set_error(S_ERR_ARG, "internal: tile list does not match variant");
+  int v = d.variant;
+  if (kF32Variants[v].nt) {
+    if (nt_usable(d, X, Y)) return launch_nt(d, X, Y, C, st);
+    v = kF32Fallback;  // same tile list (edge 20)
   }
-  SF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, dsmem));
+  SF_CUDA(cudaMemsetAsync(d.counter, 0, sizeof(unsigned int), st));
+  F32Kernel kern = f32_kernel_of(v, d.x.trans, d.y.trans);
+  const size_t smem = f32_smem(v);
+  SF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int per_sm = 0;
+  SF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kF32Warps * 32, smem));
   if (per_sm < 1) per_sm = 1;
-  int64_t want = (d.ntiles + warps - 1) / warps;
-  int grid = (int)std::min<int64_t>(want, (int64_t)num_sms() * per_sm);
-  kern<<<grid, warps * 32, dsmem, st>>>(a, (const T*)X, (const T*)Y, (T*)C);
+  const int64_t want = (d.ntiles + kF32Warps - 1) / kF32Warps;
+  const int grid = (int)std::min<int64_t>(want, (int64_t)num_sms() * per_sm);
+  kern<<<grid, kF32Warps * 32, smem, st>>>(mul_args(d), (const float*)X, (const float*)Y, (float*)C);
+  SF_CUDA(cudaGetLastError());
+  return S_OK;
+}
+
+static s_status launch_f64(const MulDesc& d, const void* X, const void* Y, void* C, cudaStream_t st) {
+  if (d.ntiles == 0) return S_OK;
+  const int edge = kF64Edges[d.variant < kNumF64Variants ? d.variant : 0];
+  if (d.edge != edge) return set_error(S_ERR_ARG, "internal: tile list does not match the double variant");
+  SF_CUDA(cudaMemsetAsync(d.counter, 0, sizeof(unsigned int), st));
+  using K = void (*)(MulArgs, int, const double*, const double*, double*);
+  K kern = d.x.trans ? (d.y.trans ? mul_f64_kernel<true, true> : mul_f64_kernel<true, false>)
+                     : (d.y.trans ? mul_f64_kernel<false, true> : mul_f64_kernel<false, false>);
+  SF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kD64Smem));
+  int per_sm = 0;
+  SF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, kD64Smem));
+  if (per_sm < 1) per_sm = 1;
+  const int64_t want = (d.ntiles + kWarps - 1) / kWarps;
+  const int grid = (int)std::min<int64_t>(want, (int64_t)num_sms() * per_sm);
+  kern<<<grid, kWarps * 32, kD64Smem, st>>>(mul_args(d), edge, (const double*)X, (const double*)Y, (double*)C);
   SF_CUDA(cudaGetLastError());
   return S_OK;
 }
@@ -1638,9 +1714,9 @@ s_status take_timeout(const MulDesc& d) {
 s_status run_mul(const MulDesc& d, s_prec prec, const void* X, const void* Y, void* C, cudaStream_t st) {
   switch (prec) {
     case S_FP64:
-      return launch_typed<double>(d, X, Y, C, st);
+      return launch_f64(d, X, Y, C, st);
     case S_FP32:
-      return launch_typed<float>(d, X, Y, C, st);
+      return launch_f32(d, X, Y, C, st);
     case S_FP64_DF:
       return launch_df(d, X, Y, C, st);
     case S_BF16X3:

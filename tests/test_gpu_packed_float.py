@@ -1,10 +1,11 @@
-"""The packed float product at the sizes where its tiles, pieces and lists change: tile edges around
+"""The packed float product and the dealt double product at the sizes where its tiles, pieces and lists change: tile edges around
 the micro-tile classes (6, 10, 12, 16, 20), blocks of several panels and several t pieces, odd
 widths (padded t pairs), and a plan whose lists exceed what it keeps, so that every product goes
 through ranges of blocks.  Against the FP64 oracle, forward and adjoint, general and symmetric.
 
 Tolerance 1e-5 relative Frobenius on uniform [-1, 1] values (float rounding 6e-8 per operation,
-about tenfold cancellation in these sums), the bound of the other random-pattern float tests."""
+about tenfold cancellation in these sums), the bound of the other random-pattern float tests; 1e-12 in
+double."""
 import numpy as np
 import pytest
 
@@ -46,6 +47,33 @@ def test_tile_and_piece_edges(sizes, fill):
     plan.adjoint(dev(dC.val, "float32"), dev(A.val, "float32"), dev(B.val, "float32"), gA, gB)
     assert rel_frob(host(gA), wA.val) <= 1e-5
     assert rel_frob(host(gB), wB.val) <= 1e-5
+
+
+@pytest.mark.parametrize("sizes", SIZES, ids=lambda s: "-".join(map(str, s)))
+@pytest.mark.parametrize("fill", [1.0, 0.4])
+def test_double_product_deals(sizes, fill):
+    # the double product deals 8, 4 or 2 lambda blocks (pieces of at most 10 or 20) to the lanes:
+    # every tile class, both tile edges, forward and both transposes; 1e-12 as the other
+    # double tests (another summation order of at most a few thousand products)
+    from paper_2211_11681_gb300 import sformat as sf
+    seed = sum(sizes) + 50
+    bsize = np.array(sizes * 6)
+    A = drop_empty(random_bcsr(bsize, fill, seed))
+    B = drop_empty(random_bcsr(bsize, fill, seed + 1, diag=False))
+    C = drop_empty(random_bcsr(bsize, fill, seed + 2, diag=False))
+    want = oprod.mul_masked(A, B, C, nthreads=8).val
+    plan = sf.Plan(pattern_of(A), pattern_of(B), pattern_of(C), "fp64")
+    for v in range(plan.num_variants()):
+        plan.set_variant(v)
+        out = dev(np.full(len(C.val), np.nan))
+        plan.mul(dev(A.val), dev(B.val), out)
+        assert rel_frob(host(out), want) <= 1e-12, v
+    dC = C.like(W.random_values(len(C.val), seed + 3))
+    wA, wB = oadj.mul_masked_adjoint(dC, A, B)
+    gA, gB = dev(np.full(len(A.val), np.nan)), dev(np.full(len(B.val), np.nan))
+    plan.adjoint(dev(dC.val), dev(A.val), dev(B.val), gA, gB)
+    assert rel_frob(host(gA), wA.val) <= 1e-12
+    assert rel_frob(host(gB), wB.val) <= 1e-12
 
 
 def test_lists_beyond_what_a_plan_keeps():
