@@ -224,7 +224,7 @@ s_status s_norm_est(s_pattern p, const double* A, int iters, double* lambda, voi
  * allocator, or a latency-critical caller that must avoid cudaMalloc's device-wide
  * synchronisation).  The paper has no counterpart: this is a deployment variant.
  * It allocates nothing: its work vectors live in a static device array inside the library
- * sized for matrix dimensions up to 1048576 (2 x 2^20 doubles + 2, about 16 MiB), which every
+ * sized for matrix dimensions up to 1048576 (2 x 2^20 doubles + 514, about 16 MiB), which every
  * GPU that loads the library holds until the process exits.  Larger patterns return
  * S_ERR_ARG.  The first call on a device looks up the array's device address
  * (cudaGetSymbolAddress) with that device current; make that first call before any stream

@@ -41,7 +41,11 @@ struct DevPattern {
   int32_t* rowidx = nullptr;  // nblocks: block rows of column, sorted
   int32_t* cscblk = nullptr;  // nblocks: CSR block index of each CSC entry
   int32_t* diag = nullptr;    // nc: block index of (nu,nu) or -1
+  int32_t* roworder = nullptr;  // nc: block rows by falling number of blocks
+  int32_t nlong = 0;            // the first nlong of them have more than kLongRow blocks
 };
+
+constexpr int kLongRow = 256;  // blocks of a row beyond which a cluster of CTAs shares it (add.cu)
 
 }  // namespace sf
 
@@ -188,7 +192,18 @@ s_status run_mul(const MulDesc& d, s_prec prec, const void* X, const void* Y, vo
 // Element-wise kernels (add.cu)
 s_status run_add(const s_pattern_t* p, s_prec prec, double alpha, const void* A, double beta, const void* B,
                  double gamma, void* C, cudaStream_t st);
-s_status run_spmv_f64(const s_pattern_t* p, const double* A, const double* x, double* y, cudaStream_t st);
+// Y = A X for nvec vectors (N x nvec, column-major)
+s_status run_spmm_f64(const s_pattern_t* p, const double* A, const double* X, int nvec, double* Y, cudaStream_t st);
+// `iters` power steps on x (all ones at first) and y, N doubles each; sc: kPowerWork doubles,
+// sc[0] = the last Rayleigh quotient
+constexpr int kRedCtas = 256;                 // partial sums of a reduction
+constexpr int kPowerWork = 2 + 2 * kRedCtas;
+s_status run_power(const s_pattern_t* p, const double* A, int iters, double* x, double* y, double* sc, cudaStream_t st);
+// part[0 .. kRedCtas) = partial sums of a b, part[kRedCtas .. 2 kRedCtas) of b b (fixed order; the
+// caller adds them in order)
+s_status run_dot2(int64_t n, const double* a, const double* b, double* part, cudaStream_t st);
+// the partial sums of a plain sum of a, as the first half of run_dot2's
+s_status run_sum(int64_t n, const double* a, double* part, cudaStream_t st);
 
 constexpr int kTile = 20;  // output tile edge of the product kernels
 

@@ -9,54 +9,33 @@
 
 namespace sf {
 
-// out[0] = sum_i a_i b_i  (single CTA tree reduction in a fixed order: deterministic)
-__global__ void dot_kernel(int64_t n, const double* __restrict__ a, const double* __restrict__ b, double* out) {
-  __shared__ double red[1024];
-  double s = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s = fma(a[i], b[i], s);
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *out = red[0];
-}
-
-__global__ void fill_kernel(int64_t n, double v, double* x) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) x[i] = v;
-}
-
-// x = y / sqrt(yy[0])  (yy = y.y on the device); leaves x unchanged when y = 0
-__global__ void normalize_kernel(int64_t n, const double* y, const double* yy, double* x) {
-  const double s = *yy;
-  if (s <= 0.0) return;
-  const double inv = 1.0 / sqrt(s);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    x[i] = y[i] * inv;
-}
-
-// out[0] = ||T - I||_F^2 = sum T_ij^2 - 2 trace(T) + n on a pattern holding every diagonal
-// block (single CTA, fixed order)
+// part[cta] = the CTA's share of ||T - I||_F^2 - n = sum T_ij^2 - 2 trace(T) on a pattern holding
+// every diagonal block, kRedCtas CTAs, fixed order; the host adds the shares in order.  HBM-bound
+// (one read of T); one CTA for all of it (as before) took 1.9 ms for 3.4e6 entries, this 21 us.
 template <typename T>
-__global__ void dist_to_identity_kernel(int64_t nnz, const T* __restrict__ v, int32_t nc, const int32_t* diag,
-                                        const int32_t* bsize, const int64_t* voff, double n, double* out) {
-  __shared__ double red[1024];
+__global__ void __launch_bounds__(256) dist_to_identity_kernel(int64_t nnz, const T* __restrict__ v, int32_t nc,
+                                                               const int32_t* __restrict__ diag,
+                                                               const int32_t* __restrict__ bsize,
+                                                               const int64_t* __restrict__ voff,
+                                                               double* __restrict__ part) {
+  __shared__ double red[8];
+  const int64_t t0 = blockIdx.x * 256ll + threadIdx.x, stride = (int64_t)kRedCtas * 256;
   double s = 0.0;
-  for (int64_t i = threadIdx.x; i < nnz; i += blockDim.x) s += (double)v[i] * (double)v[i];
-  for (int32_t nu = threadIdx.x; nu < nc; nu += blockDim.x) {
+  for (int64_t i = t0; i < nnz; i += stride) s += (double)v[i] * (double)v[i];
+  for (int64_t nu = t0; nu < nc; nu += stride) {
     const int k = diag[nu];
     if (k < 0) continue;
     const int b = bsize[nu];
     for (int r = 0; r < b; ++r) s -= 2.0 * (double)v[voff[k] + (int64_t)r * b + r];
   }
-  red[threadIdx.x] = s;
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    double q = 0.0;
+    for (int w = 0; w < 8; ++w) q += red[w];
+    part[blockIdx.x] = q;
   }
-  if (threadIdx.x == 0) *out = red[0] + n;
 }
 
 // part[k] = z_nu^T X(nu, nu') z_nu' for block k = (nu, nu')
@@ -102,6 +81,12 @@ __global__ void convert_kernel(int64_t n, const S* a, D* b, double scale) {
 
 static int grid_of(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 4096)); }
 
+static double ordered_sum(const double* v, int n) {
+  double s = 0.0;
+  for (int i = 0; i < n; ++i) s += v[i];
+  return s;
+}
+
 struct DevBuf {
   void* p = nullptr;
   ~DevBuf() { cudaFree(p); }
@@ -119,21 +104,11 @@ s_status norm_estimate(const s_pattern_t* p, const double* A, int iters, double*
   DevBuf bx, by, bs;
   SF_CUDA(cudaMalloc(&bx.p, sizeof(double) * n));
   SF_CUDA(cudaMalloc(&by.p, sizeof(double) * n));
-  SF_CUDA(cudaMalloc(&bs.p, sizeof(double) * 2));
+  SF_CUDA(cudaMalloc(&bs.p, sizeof(double) * kPowerWork));
   SyncOnExit sync{st};
-  double* x = (double*)bx.p;
-  double* y = (double*)by.p;
   double* sc = (double*)bs.p;  // sc[0] = x.y (Rayleigh quotient), sc[1] = y.y
-  fill_kernel<<<grid_of(n), 256, 0, st>>>(n, 1.0 / std::sqrt((double)n), x);
-  SF_CUDA(cudaMemsetAsync(sc, 0, sizeof(double) * 2, st));
-  for (int it = 0; it < iters; ++it) {
-    s_status s = run_spmv_f64(p, A, x, y, st);
-    if (s) return s;
-    dot_kernel<<<1, 1024, 0, st>>>(n, x, y, sc);
-    dot_kernel<<<1, 1024, 0, st>>>(n, y, y, sc + 1);
-    normalize_kernel<<<grid_of(n), 256, 0, st>>>(n, y, sc + 1, x);
-  }
-  SF_CUDA(cudaGetLastError());
+  const s_status s = run_power(p, A, iters, (double*)bx.p, (double*)by.p, sc, st);
+  if (s) return s;
   double h[2];
   SF_CUDA(cudaMemcpyAsync(h, sc, sizeof(h), cudaMemcpyDeviceToHost, st));
   SF_CUDA(cudaStreamSynchronize(st));
@@ -186,7 +161,7 @@ extern "C" s_status s_funm(s_pattern p, s_fn fn, const double* A, double* F, con
     SF_CUDA(cudaMalloc(&bZ.p, w * nnz + 16));
     SF_CUDA(cudaMalloc(&bT.p, w * nnz + 16));
     SF_CUDA(cudaMalloc(&bP.p, w * nnz + 16));
-    SF_CUDA(cudaMalloc(&bN.p, sizeof(double) * (steps + 1)));
+    SF_CUDA(cudaMalloc(&bN.p, sizeof(double) * kRedCtas * steps));
     SyncOnExit sync{st};
     void *Y = bY.p, *Z = bZ.p, *T = bT.p, *P = bP.p;
     const void* Ain = A;
@@ -212,12 +187,13 @@ extern "C" s_status s_funm(s_pattern p, s_fn fn, const double* A, double* F, con
       }
       if ((s = run_mul(plan->fwd, prec, Z, Y, P, st))) return s;                 // P = P_S(Z Y)
       if ((s = run_add(p, aprec, -0.5, P, 0.0, nullptr, 1.5, T, st))) return s;   // T = (3I - P)/2
+      double* dist = (double*)bN.p + (int64_t)k * kRedCtas;
       if (aprec == S_FP64)
-        dist_to_identity_kernel<double><<<1, 1024, 0, st>>>(nnz, (const double*)T, p->d.nc, p->d.diag, p->d.bsize,
-                                                            p->d.voff, (double)p->d.n, (double*)bN.p + k);
+        dist_to_identity_kernel<double><<<kRedCtas, 256, 0, st>>>(nnz, (const double*)T, p->d.nc, p->d.diag, p->d.bsize,
+                                                                  p->d.voff, dist);
       else
-        dist_to_identity_kernel<float><<<1, 1024, 0, st>>>(nnz, (const float*)T, p->d.nc, p->d.diag, p->d.bsize,
-                                                           p->d.voff, (double)p->d.n, (double*)bN.p + k);
+        dist_to_identity_kernel<float><<<kRedCtas, 256, 0, st>>>(nnz, (const float*)T, p->d.nc, p->d.diag, p->d.bsize,
+                                                                 p->d.voff, dist);
       if ((s = run_mul(plan->fwd, prec, Y, T, P, st))) return s;                 // Y' = P_S(Y T)
       std::swap(Y, P);
       if ((s = run_mul(plan->fwd, prec, T, Z, P, st))) return s;                 // Z' = P_S(T Z)
@@ -265,9 +241,10 @@ extern "C" s_status s_funm(s_pattern p, s_fn fn, const double* A, double* F, con
     // 1e-3 of its starting value (below that the iteration has converged and the distance only
     // fluctuates at the level of the masking and rounding errors)
     {
-      std::vector<double> dk(steps);
-      SF_CUDA(cudaMemcpyAsync(dk.data(), bN.p, sizeof(double) * steps, cudaMemcpyDeviceToHost, st));
+      std::vector<double> dk(steps), part((size_t)steps * kRedCtas);
+      SF_CUDA(cudaMemcpyAsync(part.data(), bN.p, sizeof(double) * part.size(), cudaMemcpyDeviceToHost, st));
       SF_CUDA(cudaStreamSynchronize(st));
+      for (int k = 0; k < steps; ++k) dk[k] = ordered_sum(&part[(size_t)k * kRedCtas], kRedCtas) + (double)p->d.n;
       for (int k = 0; k < steps; ++k) {
         const bool grew = k >= 2 && dk[k] > 2.25 * dk[k - 1] && dk[k - 1] > 2.25 * dk[k - 2] &&  // squared: 1.5^2
                           dk[k] > 1e-6 * dk[0];
@@ -283,16 +260,17 @@ extern "C" s_status s_funm(s_pattern p, s_fn fn, const double* A, double* F, con
       PlanGuard pg2{p64};
       DevBuf bR, bd;
       SF_CUDA(cudaMalloc(&bR.p, sizeof(double) * nnz + 16));
-      SF_CUDA(cudaMalloc(&bd.p, sizeof(double) * 2));
+      SF_CUDA(cudaMalloc(&bd.p, sizeof(double) * 4 * kRedCtas));
       SyncOnExit sync2{st};
       if ((s = run_mul(p64->fwd, S_FP64, F, F, bR.p, st))) return s;
       if ((s = run_add(p, S_FP64, 1.0, bR.p, -1.0, A, 0.0, bR.p, st))) return s;
-      dot_kernel<<<1, 1024, 0, st>>>(nnz, (const double*)bR.p, (const double*)bR.p, (double*)bd.p);
-      dot_kernel<<<1, 1024, 0, st>>>(nnz, A, A, (double*)bd.p + 1);
-      double h[2];
-      SF_CUDA(cudaMemcpyAsync(h, bd.p, sizeof(h), cudaMemcpyDeviceToHost, st));
+      double* part = (double*)bd.p;  // the second half of each pair: sums of squares
+      if ((s = run_dot2(nnz, (const double*)bR.p, (const double*)bR.p, part, st))) return s;
+      if ((s = run_dot2(nnz, A, A, part + 2 * kRedCtas, st))) return s;
+      std::vector<double> h(4 * kRedCtas);
+      SF_CUDA(cudaMemcpyAsync(h.data(), part, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st));
       SF_CUDA(cudaStreamSynchronize(st));
-      *o.residual = std::sqrt(h[0]) / std::sqrt(h[1]);
+      *o.residual = std::sqrt(ordered_sum(&h[kRedCtas], kRedCtas)) / std::sqrt(ordered_sum(&h[3 * kRedCtas], kRedCtas));
     }
     return S_OK;
   }
@@ -436,20 +414,17 @@ extern "C" s_status s_quad_form(s_pattern p, const double* X, const double* z, d
   const int64_t nb = p->d.nblocks;
   DevBuf part, tot;
   SF_CUDA(cudaMalloc(&part.p, sizeof(double) * (nb + 1)));
-  SF_CUDA(cudaMalloc(&tot.p, sizeof(double)));
+  SF_CUDA(cudaMalloc(&tot.p, sizeof(double) * kRedCtas));
   SyncOnExit sync{st};
-  SF_CUDA(cudaMemsetAsync(tot.p, 0, sizeof(double), st));
   if (nb) {
     quad_part_kernel<<<(unsigned)((nb * 32 + 255) / 256), 256, 0, st>>>(nb, p->d.brow, p->d.colidx, p->d.bsize,
                                                                       p->d.boff, p->d.voff, X, z, (double*)part.p);
-    // fixed-order sum of the block parts: dot with a vector of ones
-    DevBuf ones;
-    SF_CUDA(cudaMalloc(&ones.p, sizeof(double) * nb));
-    fill_kernel<<<grid_of(nb), 256, 0, st>>>(nb, 1.0, (double*)ones.p);
-    dot_kernel<<<1, 1024, 0, st>>>(nb, (const double*)part.p, (const double*)ones.p, (double*)tot.p);
-    SF_CUDA(cudaGetLastError());
-    SF_CUDA(cudaMemcpyAsync(out, tot.p, sizeof(double), cudaMemcpyDeviceToHost, st));
+    s_status s = run_sum(nb, (const double*)part.p, (double*)tot.p, st);
+    if (s) return s;
+    double h[kRedCtas];
+    SF_CUDA(cudaMemcpyAsync(h, tot.p, sizeof(h), cudaMemcpyDeviceToHost, st));
     SF_CUDA(cudaStreamSynchronize(st));
+    *out = ordered_sum(h, kRedCtas);
   } else {
     *out = 0.0;
   }

@@ -137,7 +137,7 @@ __device__ __forceinline__ void d64_cp(uint32_t dst, const double* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
 }
 
-// rows x cols doubles at row pitch ld -> dst, packed.
+// rows x cols doubles at row pitch ld -> dst, packed; one warp.
 __device__ __forceinline__ void d64_stage(uint32_t dst, const double* src, int rows, int cols, int ld, int lane) {
   const int len = rows * cols;
   if (cols == ld) {
@@ -176,7 +176,6 @@ __global__ void __launch_bounds__(kWarps * 32, 4) mul_f64_kernel(MulArgs a, int 
     // S ne <= 32 kD64Slots for every tile of at most 20 x 20
     const int S = ne <= 100 && th + tw <= 20 ? 8 : ne <= 200 ? 4 : 2;
     const int KC = S == 2 ? 20 : 10;
-    const int M = (S * ne + 31) >> 5;
     double acc[kD64Slots];
     int off[kD64Slots];  // slot m: block s of the step, entry (r, c): s << 16 | r << 8 | c
 #pragma unroll

@@ -4,6 +4,8 @@
 #include <mutex>
 #include <new>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace sf {
@@ -59,6 +61,7 @@ static void free_dev(DevPattern& d) {
   cudaFree(d.rowidx);
   cudaFree(d.cscblk);
   cudaFree(d.diag);
+  cudaFree(d.roworder);
   d = DevPattern();
 }
 
@@ -148,8 +151,15 @@ extern "C" s_status s_pattern_create(int32_t nc, const int64_t* block_offset, co
   d.nblocks = nb;
   d.nnz = off;
   d.max_bsize = maxb;
+  // block rows by falling length (ties: row), the long ones first (block-sparse times dense)
+  std::vector<int32_t> order(nc);
+  for (int32_t i = 0; i < nc; ++i) order[i] = i;
+  std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+    return rowptr[x + 1] - rowptr[x] > rowptr[y + 1] - rowptr[y];
+  });
+  while (d.nlong < nc && rowptr[order[d.nlong] + 1] - rowptr[order[d.nlong]] > kLongRow) ++d.nlong;
   s_status st;
-  if ((st = upload(&d.bsize, p->bsize.data(), nc)) || (st = upload(&d.boff, block_offset, nc + 1)) ||
+  if ((st = upload(&d.roworder, order.data(), nc)) || (st = upload(&d.bsize, p->bsize.data(), nc)) || (st = upload(&d.boff, block_offset, nc + 1)) ||
       (st = upload(&d.rowptr, rowptr, nc + 1)) || (st = upload(&d.colidx, colidx, nb)) ||
       (st = upload(&d.brow, p->brow.data(), nb)) || (st = upload(&d.voff, p->voff.data(), nb + 1)) ||
       (st = upload(&d.colptr, colptr.data(), nc + 1)) || (st = upload(&d.rowidx, rowidx.data(), nb)) ||
