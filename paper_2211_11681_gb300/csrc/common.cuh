@@ -162,6 +162,7 @@ struct MulDesc {
   NtTile* nt_tiles = nullptr;      // tiles of S_C in block order
   NtEntry* nt_ent = nullptr;       // lists of the current range (nullptr: side or lists missing)
   std::vector<NtRange> nt_ranges;  // one: the plan keeps all lists
+  int nt_per_sm = 1;               // resident CTAs of the packed kernel
   bool nt_ysym = false;            // Y side read through X's rows (B = A, symmetric)
   float2* df_x = nullptr;    // S_FP64_DF: split operands (hi, lo)
   float2* df_y = nullptr;
@@ -206,6 +207,35 @@ s_status run_dot2(int64_t n, const double* a, const double* b, double* part, cud
 s_status run_sum(int64_t n, const double* a, double* part, cudaStream_t st);
 
 constexpr int kTile = 20;  // output tile edge of the product kernels
+
+// Asynchronous copies global -> shared of 8 and 16 bytes.
+__device__ __forceinline__ void d64_cp(uint32_t dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void d64_cp2(uint32_t dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+}
+
+// rows x cols doubles at row pitch ld -> dst, packed; one warp.  A packed source on 16-byte
+// boundaries goes two doubles to a copy.
+__device__ __forceinline__ void d64_stage(uint32_t dst, const double* src, int rows, int cols, int ld, int lane) {
+  const int len = rows * cols;
+  if (cols == ld) {
+    if (((dst | (uint32_t)reinterpret_cast<uintptr_t>(src)) & 15) == 0) {
+      for (int e = 2 * lane; e + 1 < len; e += 64) d64_cp2(dst + 8u * (uint32_t)e, src + e);
+      if ((len & 1) && lane == 0) d64_cp(dst + 8u * (uint32_t)(len - 1), src + len - 1);
+    } else {
+#pragma unroll 4
+      for (int e = lane; e < len; e += 32) d64_cp(dst + 8u * (uint32_t)e, src + e);
+    }
+  } else {
+    const float rc = 1.0f / (float)cols;
+    for (int e = lane; e < len; e += 32) {
+      const int r = __float2int_rz(((float)e + 0.5f) * rc);
+      d64_cp(dst + 8u * (uint32_t)e, src + (int64_t)r * ld + (e - r * cols));
+    }
+  }
+}
 
 }  // namespace sf
 

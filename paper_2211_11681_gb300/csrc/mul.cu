@@ -132,26 +132,6 @@ struct D64Entry {
   uint16_t t0, kc; // first t and t extent of this piece
 };
 
-// 8-byte asynchronous copy global -> shared.
-__device__ __forceinline__ void d64_cp(uint32_t dst, const double* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
-}
-
-// rows x cols doubles at row pitch ld -> dst, packed; one warp.
-__device__ __forceinline__ void d64_stage(uint32_t dst, const double* src, int rows, int cols, int ld, int lane) {
-  const int len = rows * cols;
-  if (cols == ld) {
-#pragma unroll 4
-    for (int e = lane; e < len; e += 32) d64_cp(dst + 8u * (uint32_t)e, src + e);
-  } else {
-    const float rc = 1.0f / (float)cols;
-    for (int e = lane; e < len; e += 32) {
-      const int r = __float2int_rz(((float)e + 0.5f) * rc);
-      d64_cp(dst + 8u * (uint32_t)e, src + (int64_t)r * ld + (e - r * cols));
-    }
-  }
-}
-
 template <bool TX, bool TY>
 __global__ void __launch_bounds__(kWarps * 32, 4) mul_f64_kernel(MulArgs a, int edge, const double* __restrict__ X,
                                                                  const double* __restrict__ Y, double* __restrict__ C) {
@@ -178,11 +158,13 @@ __global__ void __launch_bounds__(kWarps * 32, 4) mul_f64_kernel(MulArgs a, int 
     const int KC = S == 2 ? 20 : 10;
     double acc[kD64Slots];
     int off[kD64Slots];  // slot m: block s of the step, entry (r, c): s << 16 | r << 8 | c
+    const float rne = 1.0f / (float)ne, rtw = 1.0f / (float)tw;
 #pragma unroll
     for (int m = 0; m < kD64Slots; ++m) {
       acc[m] = 0.0;
       const int i = min(lane + 32 * m, S * ne - 1);
-      const int s = i / ne, e = i - s * ne, r = e / tw;
+      const int s = __float2int_rz(((float)i + 0.5f) * rne), e = i - s * ne;
+      const int r = __float2int_rz(((float)e + 0.5f) * rtw);
       off[m] = s << 16 | r << 8 | (e - r * tw);
     }
     const int px1 = (int)a.x.ptr[nu + 1];
@@ -271,7 +253,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) mul_f64_kernel(MulArgs a, int 
     for (int e = lane; e < ne; e += 32) {
       double v = base[e];
       for (int s = 1; s < S; ++s) v += base[s * ne + e];
-      const int r = e / tw, c = e - r * tw;
+      const int r = __float2int_rz(((float)e + 0.5f) * rtw), c = e - r * tw;
       cb[(int64_t)r * nj + c] = v;
     }
     __syncwarp();

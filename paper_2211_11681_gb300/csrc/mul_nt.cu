@@ -361,27 +361,38 @@ __global__ void __launch_bounds__(kNtWarps * 32, 4) mul_f32_nt_kernel(NtArgs a) 
   }
 }
 
-// Packed copy of a pattern's blocks: block b (rows x cols, row-major in `src` at voff[b]), or its
+// One operand of the pre-pass: its blocks as stored and where the packed ones go.
+struct NtPack {
+  int64_t nb;
+  const int32_t* bsize;
+  const int32_t* brow;
+  const int32_t* bcol;
+  const int64_t* voff;
+  const int64_t* poff;
+  int trans;
+  const float* src;
+  float* dst;
+};
+
+// Blocks w0, w0 + nw, .. of an operand: block b (rows x cols, row-major in `src` at voff[b]), or its
 // transpose (trans), is written at poff[b] as panels of at most 20 rows, [t / 2][row][t % 2] each,
-// zeros for the padded t and up to the next multiple of 4 floats.  One warp per block; a lane
+// zeros for the padded t and up to the next multiple of 4 floats.  kNtPackLanes lanes per block
+// (a chain of dependent loads leads to each block: 8 lanes keep 4 blocks of a warp in flight); a lane
 // writes one pair of t (8 bytes) at a time.
-__global__ void nt_prepare_kernel(int64_t nb, const int32_t* __restrict__ bsize, const int32_t* __restrict__ brow,
-                                  const int32_t* __restrict__ bcol, const int64_t* __restrict__ voff,
-                                  const int64_t* __restrict__ poff, int trans, const float* __restrict__ src,
-                                  float* __restrict__ dst) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; b < nb;
-       b += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int rows = bsize[brow[b]], cols = bsize[bcol[b]];
-    const int R = trans ? cols : rows, K = trans ? rows : cols;  // panel rows and t extent
-    const int rs = trans ? 1 : cols, ts = trans ? cols : 1;      // source strides of a row and of t
+constexpr int kNtPackLanes = 8;
+__device__ __forceinline__ void nt_pack(const NtPack& p, int64_t w0, int64_t nw, int lane) {
+  for (int64_t b = w0; b < p.nb; b += nw) {
+    const int rows = p.bsize[p.brow[b]], cols = p.bsize[p.bcol[b]];
+    const int R = p.trans ? cols : rows, K = p.trans ? rows : cols;  // panel rows and t extent
+    const int rs = p.trans ? 1 : cols, ts = p.trans ? cols : 1;      // source strides of a row and of t
     const int kp = nt_even(K) >> 1;
-    const float* s = src + voff[b];
-    float2* d = reinterpret_cast<float2*>(dst + poff[b]);
+    const float* __restrict__ s = p.src + p.voff[b];
+    float2* __restrict__ d = reinterpret_cast<float2*>(p.dst + p.poff[b]);
     for (int r0 = 0; r0 < R; r0 += kTile) {
       const int th = min(kTile, R - r0);
       const float rth = 1.0f / (float)th;
-      for (int e = lane; e < th * kp; e += 32) {
+#pragma unroll 4
+      for (int e = lane; e < th * kp; e += kNtPackLanes) {
         const int tp = e < (1 << 20) ? __float2int_rz(((float)e + 0.5f) * rth) : e / th, r = r0 + e - tp * th;
         const float* v = s + (int64_t)r * rs + (int64_t)(2 * tp) * ts;
         d[(int64_t)r0 * kp + e] = make_float2(v[0], 2 * tp + 1 < K ? v[ts] : 0.0f);
@@ -389,6 +400,17 @@ __global__ void nt_prepare_kernel(int64_t nb, const int32_t* __restrict__ bsize,
     }
     if (lane == 0 && ((R * kp) & 1)) d[(int64_t)R * kp] = make_float2(0.0f, 0.0f);
   }
+}
+
+// Packed copies of both operands (y.nb = 0: one copy serves both sides), and zero in the product's
+// tile counter: small products are bound by their launches.
+__global__ void nt_prepare_kernel(NtPack x, NtPack y, unsigned int* counter) {
+  const int lane = threadIdx.x % kNtPackLanes;
+  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kNtPackLanes;
+  const int64_t nw = (int64_t)gridDim.x * blockDim.x / kNtPackLanes;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0u;
+  nt_pack(x, w, nw, lane);
+  nt_pack(y, w, nw, lane);
 }
 
 }  // namespace
@@ -460,6 +482,9 @@ void nt_free_lists(MulDesc* d) {
 // on the tile kernel.  All work is on the default stream and finished on return.
 static s_status nt_build_lists(MulDesc* d) {
   nt_free_lists(d);
+  SF_CUDA(cudaFuncSetAttribute(mul_f32_nt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNtSmem));
+  SF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d->nt_per_sm, mul_f32_nt_kernel, kNtWarps * 32, kNtSmem));
+  d->nt_per_sm = std::max(d->nt_per_sm, 1);
   if (!d->ntx.off || !d->nty.off) return S_OK;
   // the entries count operand offsets in 4 floats with 32 bits, t in 16
   if ((d->ntx.len >> 2) > (int64_t)UINT32_MAX || (d->nty.len >> 2) > (int64_t)UINT32_MAX) return S_OK;
@@ -564,14 +589,9 @@ s_status nt_configure(MulDesc* d, bool x_trans, bool y_trans, bool y_sym) {
   return nt_build_lists(d);
 }
 
-static s_status nt_prepare(const NtSideDesc& s, const float* src, cudaStream_t st) {
+static NtPack pack_of(const NtSideDesc& s, const void* src) {
   const DevPattern& p = s.pat->d;
-  if (p.nblocks == 0) return S_OK;
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((p.nblocks * 32 + 255) / 256, (int64_t)sm_count() * 16));
-  nt_prepare_kernel<<<grid, 256, 0, st>>>(p.nblocks, p.bsize, p.brow, p.colidx, p.voff, s.poff, s.trans ? 1 : 0, src,
-                                          s.scratch);
-  SF_CUDA(cudaGetLastError());
-  return S_OK;
+  return NtPack{p.nblocks, p.bsize, p.brow, p.colidx, p.voff, s.poff, s.trans ? 1 : 0, (const float*)src, s.scratch};
 }
 
 bool nt_usable(const MulDesc& d, const void* X, const void* Y) {
@@ -584,13 +604,11 @@ s_status launch_nt(const MulDesc& d, const void* X, const void* Y, void* C, cuda
   if (d.ntiles == 0) return S_OK;
   s_status s = take_timeout(d);
   if (s) return s;
-  if ((s = nt_prepare(d.ntx, (const float*)X, st))) return s;
-  if (!d.nty.from_x && (s = nt_prepare(d.nty, (const float*)Y, st))) return s;
-  void (*kern)(NtArgs) = mul_f32_nt_kernel;
-  SF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNtSmem));
-  int per_sm = 0;
-  SF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kNtWarps * 32, kNtSmem));
-  if (per_sm < 1) per_sm = 1;
+  const NtPack px = pack_of(d.ntx, X);
+  const NtPack py = d.nty.from_x ? NtPack{} : pack_of(d.nty, Y);
+  const int64_t ctas = (std::max(px.nb, py.nb) * kNtPackLanes + 255) / 256;
+  nt_prepare_kernel<<<(int)std::max<int64_t>(1, std::min<int64_t>(ctas, (int64_t)sm_count() * 16)), 256, 0, st>>>(
+      px, py, d.counter);
   const DevPattern& pc = d.pc->d;
   for (const NtRange& r : d.nt_ranges) {
     if (d.nt_ranges.size() > 1) {
@@ -607,10 +625,10 @@ s_status launch_nt(const MulDesc& d, const void* X, const void* Y, void* C, cuda
     a.ntiles = (uint32_t)(r.t1 - r.t0);
     a.counter = d.counter;
     a.C = (float*)C;
-    SF_CUDA(cudaMemsetAsync(d.counter, 0, sizeof(unsigned int), st));
+    if (r.k0 > 0) SF_CUDA(cudaMemsetAsync(d.counter, 0, sizeof(unsigned int), st));
     const int64_t want = (r.t1 - r.t0 + kNtWarps - 1) / kNtWarps;
-    const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count() * per_sm);
-    if (grid > 0) kern<<<grid, kNtWarps * 32, kNtSmem, st>>>(a);
+    const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count() * d.nt_per_sm);
+    if (grid > 0) mul_f32_nt_kernel<<<grid, kNtWarps * 32, kNtSmem, st>>>(a);
     SF_CUDA(cudaGetLastError());
   }
   return S_OK;
