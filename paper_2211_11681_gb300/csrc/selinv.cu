@@ -13,30 +13,32 @@
 //             both row i and row k of L;
 //     pivot   D(k,k) = W(k,k) inverted by Gauss-Jordan in shared memory (positive definite:
 //             no pivoting; a pivot that is not positive is recorded), then
-//             L(i,k) = W(i,k) D(k,k)^{-1} for the blocks of column k (a CTA per supernode
-//             and slice of its column), D^{-1} stored in L's diagonal block;
+//             L(i,k) = W(i,k) D(k,k)^{-1} for the rows of column k (a CTA per supernode
+//             and range of rows), D^{-1} stored in L's diagonal block;
 //   inversion, levels from the root down (Takahashi-type recurrences from Eq. (blockInv)):
 //     off     Z(i,k) = - sum_{j in struct(k)} Z(i,j) L(j,k), Z(i,j) read from block
 //             (max, min) of Z, transposed when i < j;
-//     diag    Z(k,k) = D(k,k)^{-1} - sum_{j in struct(k)} Z(j,k)^T L(j,k) (a CTA per
-//             supernode, its warps splitting the sum);
+//     diag    Z(k,k) = D(k,k)^{-1} - sum_{j in struct(k)} Z(j,k)^T L(j,k) (a CTA or a cluster of
+//             CTAs per supernode, its warps splitting the sum);
 //   scatter   out = alpha P_S(Z) + beta out, blocks of S read from Z or its transpose.
 //
 // The terms of every sum are fixed by the pattern of L, so the plan lists them once (the
 // symbolic phase of both sweeps): per block of L the pairs (W(i,j), L(k,j)) of the update and
-// (Z(i,j), L(j,k)) of the inversion.  The update and off-diagonal steps give one warp an
-// output block (512-entry tiles of it, 16 entries per lane) and a contiguous part of its
-// term list: near the root the elimination tree is a chain whose levels hold few, long sums,
-// so the host splits each list into `split` parts (split-K) to keep every SM sub-partition
-// busy.  With split > 1 the parts land in a scratch buffer and the next launch of the level
-// (pivot, diag) adds them in a fixed order, so results do not depend on scheduling.  The
-// operand blocks of each term are staged in shared memory 16 columns at a time (row pitch 17
-// doubles: rows fall in different banks) by cp.async into one of two buffers per warp, the
-// next unit's copies in flight while the current unit is multiplied.
+// (Z(i,j), L(j,k)) of the inversion.  A warp sums a tile of at most 20 x 20 entries of one output
+// block over a part of its list, 8, 4 or 2 terms at a time dealt to its lanes as in the double
+// product (si_sum): the FP64 pipe takes as long for 1 lane as for 32.  Near the root the
+// elimination tree is a chain whose levels hold few, long sums, so the host splits each list
+// over the 4 warps of a CTA and, where that leaves SMs idle, over several CTAs (split-K): the
+// warps' sums are added in the CTA, the CTAs' parts land in a scratch buffer and the next
+// launch of the level (pivot, diag) adds them, all in a fixed order, so results do not depend
+// on scheduling.  What bounds a level is its chain of latencies (term list, operand offsets, copies,
+// at least 8 terms' FP64 instructions) more than its operations; see the kernels.
 //
 // Every entry a launch reads was written by an earlier launch (descendants sit on lower
 // levels, ancestors on higher ones) or by its own CTA before a barrier, so the kernels need
 // no synchronisation beyond stream order and no waits.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -50,21 +52,21 @@ namespace sf {
 namespace {
 
 constexpr int kSiMaxB = 64;               // widest block
-constexpr int kSiEnt = 16;                // output entries per lane
-constexpr int kSiTileEnt = 32 * kSiEnt;   // entries of one work item
-constexpr int kSiWarps = 4;               // warps per CTA of the block kernels
-constexpr int kSiThreads = 128;           // threads of the pivot and diagonal kernels
-constexpr int kSiSlice = 8;               // column blocks per pivot CTA
-constexpr int kSiU = 16;                  // columns of t staged per slice
-constexpr int kSiUp = kSiU + 1;           // row pitch of a staged slice (doubles)
-constexpr int kSiMaxSplit = 64;           // parts of one split sum
-constexpr int kSiPartTerms = 4;           // fewest terms of one part
+constexpr int kSiWarps = 4;               // warps per CTA of the sum kernels
+constexpr int kSiThreads = 256;           // threads of the pivot kernel
+constexpr int kSiSlots = 25;              // accumulators of a lane
+constexpr int kSiChains = 2;              // accumulators a full step works on at a time
+constexpr int kSiBuf = 1600;              // doubles of a warp's stage buffer
+constexpr int kSiChunk = 2048;            // doubles of W a pivot CTA holds at a time
+constexpr int kSiCluster = 8;             // CTAs that share a long diagonal sum
+constexpr int kSiStepTerms = 2;           // fewest terms worth a warp
+constexpr int kSiMaxParts = 16;           // CTAs of one split sum
 constexpr int kSiMaxClusters = 32768;     // non-empty clusters of the host bitset analysis
 
 struct SiItem {
-  int32_t blk;  // CSC block of L
-  int32_t col;  // its column position
-  int32_t e0;   // first entry of the tile
+  int32_t blk;      // CSC block of L
+  int32_t col;      // its column position
+  int16_t r0, c0;   // tile of at most kTile x kTile entries
 };
 
 struct SiDev {
@@ -87,381 +89,328 @@ struct SiDev {
   double* Z;              // the inverse on the pattern of L
   double* P;              // partial sums of split launches: [part][entries of the level]
   unsigned int* flag;     // mapped host word: 1 = a pivot block was not positive definite
-  int maxb;               // widest block of the plan
 };
 
-// Entry coordinates of a lane's kSiEnt entries of a rows x cols tile starting at e0.
-__device__ __forceinline__ void si_entries(int e0, int ne, int cols, int lane, int* rr, int* cc) {
+// Which terms a sum runs over: the update's list, the inversion's list, or the blocks of column k.
+enum { kSiUpdate, kSiOff, kSiDiag };
+
+// One warp's sum over terms t .. te-1 (t steps of S) of a th x tw tile: sum of x(r0 + r, :) y(:, c0 + c).
+// On return base[e] (e = r tw + c) holds the sum.  The operands of S terms are staged together
+// and their (term, entry) pairs dealt to the lanes, kSiSlots accumulators each (the rules of
+// mul_f64_kernel).  Blocks are staged in the order they are stored; the next terms' offsets are
+// fetched while the copies arrive.
+template <int MODE>
+__device__ __forceinline__ void si_sum(const SiDev& s, int64_t t, int64_t te, int64_t q0, int bi, int bk, int r0, int c0,
+                                       int th, int tw, double* base, int lane) {
+  constexpr bool kYRows = MODE == kSiUpdate;  // y stored [c][t] (L(k,j)), else [t][c] (L(j,k))
+  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(base);
+  const int ne = th * tw;
+  const int S = ne <= 100 && th + tw <= 20 ? 8 : ne <= 200 ? 4 : 2;
+  const int KC = S == 2 ? 20 : 10;
+  double acc[kSiSlots];
+  int off[kSiSlots];  // slot m: term s of the step, entry (r, c): s << 16 | r << 8 | c
+  const float rne = 1.0f / (float)ne, rtw = 1.0f / (float)tw;
+  const int used = (int)max((int64_t)0, min((int64_t)S, te - t)) * ne;  // (term, entry) pairs of a step at most
 #pragma unroll
-  for (int m = 0; m < kSiEnt; ++m) {
-    const int e = e0 + lane + 32 * m;
-    rr[m] = e < ne ? e / cols : -1;
-    cc[m] = e < ne ? e - rr[m] * cols : 0;
+  for (int m = 0; m < kSiSlots; ++m) {
+    acc[m] = 0.0;
+    off[m] = 0;
+    if (32 * m >= used) continue;
+    const int i = min(lane + 32 * m, used - 1);
+    const int u = __float2int_rz(((float)i + 0.5f) * rne), e = i - u * ne;
+    const int r = __float2int_rz(((float)e + 0.5f) * rtw);
+    off[m] = u << 16 | r << 8 | (e - r * tw);
   }
-}
-
-// acc[m] += sign * sum_t a[rr[m]][t] b[cc[m]][t] over t < uw (staged slices).
-__device__ __forceinline__ void si_dot(const double* a, const double* b, int uw, const int* rr, const int* cc,
-                                       double sign, double* acc) {
+  // lane u holds term u of the next step: t extent (0: none; negative: x is stored transposed) and
+  // where its operands start
+  int nj = 0;
+  int64_t nx = 0, ny = 0;
+  auto fetch = [&](int64_t from) {
+    nj = 0;
+    const int64_t q = from + lane;
+    if (lane >= S || q >= te) return;
+    if (MODE == kSiUpdate) {
+      const int bw = s.uw[q];
+      nj = s.bs[s.colcol[bw]];
+      nx = s.loff[bw];
+      ny = s.loff[s.ul[q]];
+    } else if (MODE == kSiOff) {
+      const int zb = s.oz[q], qq = s.ol[q];
+      nj = s.bs[s.colrow[qq]];
+      nx = s.loff[zb < 0 ? ~zb : zb];
+      if (zb < 0) nj = -nj;
+      ny = s.loff[qq];
+    } else {
+      nj = -s.bs[s.colrow[q0 + q]];
+      nx = ny = s.loff[q0 + q];
+    }
+  };
+  const double* xall = MODE == kSiUpdate ? s.W : s.Z;
+  fetch(t);
+  for (; t < te; t += S) {
+    const int n = (int)min((int64_t)S, te - t);
+    const int mj = nj;
+    const int64_t mx = nx, my = ny;
+    const int widest = (int)__reduce_max_sync(0xffffffffu, (unsigned)abs(mj));
+    for (int t0 = 0; t0 < widest; t0 += KC) {
+      const int kc = min(KC, widest - t0), sx = th * kc, ss = sx + kc * tw;
+      __syncwarp();
+      for (int u = 0; u < n; ++u) {
+        const int sj = __shfl_sync(0xffffffffu, mj, u), bj = abs(sj);
+        const int64_t xo = __shfl_sync(0xffffffffu, mx, u), yo = __shfl_sync(0xffffffffu, my, u);
+        const int kw = min(kc, bj - t0);
+        if (kw <= 0) continue;
+        const uint32_t d = sbase + 8u * (uint32_t)(u * ss);
+        if (sj < 0) d64_stage(d, xall + xo + (int64_t)t0 * bi + r0, kw, th, bi, lane);
+        else d64_stage(d, xall + xo + (int64_t)r0 * bj + t0, th, kw, bj, lane);
+        if (kYRows) d64_stage(d + 8u * (uint32_t)sx, s.L + yo + (int64_t)c0 * bj + t0, tw, kw, bj, lane);
+        else d64_stage(d + 8u * (uint32_t)sx, s.L + yo + (int64_t)t0 * bk + c0, kw, tw, bk, lane);
+      }
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+      if (t0 == 0) fetch(t + S);
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+      __syncwarp();
+      const int left = abs(mj) - t0;  // t extent left of this lane's term
+      if (n * ne == used && __all_sync(0xffffffffu, lane >= n || left >= kc)) {
+        // a full step of terms all as wide as the step: kSiChains slots' chains side by side
+        const int live = (n * ne + 31) >> 5;
 #pragma unroll
-  for (int m = 0; m < kSiEnt; ++m) {
-    if (rr[m] < 0) continue;
-    const double* ar = a + rr[m] * kSiUp;
-    const double* br = b + cc[m] * kSiUp;
-    double t0 = 0.0, t1 = 0.0;
-    int t = 0;
-    for (; t + 4 <= uw; t += 4) {
-      t0 = fma(ar[t], br[t], t0);
-      t1 = fma(ar[t + 1], br[t + 1], t1);
-      t0 = fma(ar[t + 2], br[t + 2], t0);
-      t1 = fma(ar[t + 3], br[t + 3], t1);
-    }
-    for (; t < uw; ++t) t0 = fma(ar[t], br[t], t0);
-    acc[m] = fma(sign, t0 + t1, acc[m]);
-  }
-}
-
-// Stage rows x uw values into dst[r * kSiUp + t] (zero padded to uw4 columns):
-// value(r, t) = src[r * rs + t * ts] (rs, ts: the source's row and column strides).  Plain
-// (coherent) loads: the diagonal kernel reads blocks its own CTA wrote before a barrier.
-__device__ __forceinline__ void si_stage(double* dst, const double* src, int rows, int uw, int uw4, int rs, int ts,
-                                         int lane) {
-  if (ts == 1) {
-    for (int idx = lane; idx < rows * uw4; idx += 32) {
-      const int r = idx / uw4, t = idx - r * uw4;
-      dst[r * kSiUp + t] = t < uw ? src[(int64_t)r * rs + t] : 0.0;
-    }
-  } else {
-    for (int idx = lane; idx < rows * uw4; idx += 32) {  // rows fastest: coalesced when rs = 1
-      const int t = idx / rows, r = idx - t * rows;
-      dst[r * kSiUp + t] = t < uw ? src[(int64_t)t * ts + (int64_t)r * rs] : 0.0;
-    }
-  }
-}
-
-// Asynchronous 8-byte copy global -> shared (cp.async, zero fill when !valid; src must still
-// point into the buffer), and its group commit / wait.
-__device__ __forceinline__ void si_cp8(double* dst, const double* src, bool valid) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 8 : 0) : "memory");
-}
-__device__ __forceinline__ void si_cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void si_cp_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-__device__ __forceinline__ void si_cp_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// si_stage with cp.async: the copies complete at the lane's next wait on their group.
-__device__ __forceinline__ void si_stage_async(double* dst, const double* src, int rows, int uw, int uw4, int rs,
-                                               int ts, int lane) {
-  if (ts == 1) {
-    for (int idx = lane; idx < rows * uw4; idx += 32) {
-      const int r = idx / uw4, t = idx - r * uw4;
-      si_cp8(dst + r * kSiUp + t, t < uw ? src + (int64_t)r * rs + t : src, t < uw);
-    }
-  } else {
-    for (int idx = lane; idx < rows * uw4; idx += 32) {
-      const int t = idx / rows, r = idx - t * rows;
-      si_cp8(dst + r * kSiUp + t, t < uw ? src + (int64_t)t * ts + (int64_t)r * rs : src, t < uw);
+        for (int m0 = 0; m0 < kSiSlots; m0 += kSiChains) {
+          if (m0 >= live) break;
+          const double* xp[kSiChains];
+          const double* yp[kSiChains];
+          int xt[kSiChains];
+#pragma unroll
+          for (int v = 0; v < kSiChains; ++v) {
+            const int o = off[min(m0 + v, kSiSlots - 1)], u = o >> 16, r = (o >> 8) & 255, c = o & 255;
+            const bool tr = __shfl_sync(0xffffffffu, mj, u) < 0;
+            xp[v] = base + u * ss + (tr ? r : r * kc);
+            yp[v] = base + u * ss + sx + (kYRows ? c * kc : c);
+            xt[v] = tr ? th : 1;
+          }
+#pragma unroll 2
+          for (int tt = 0; tt < kc; ++tt) {
+#pragma unroll
+            for (int v = 0; v < kSiChains; ++v) {
+              if (m0 + v < kSiSlots && m0 + v < live) acc[m0 + v] = fma(*xp[v], *yp[v], acc[m0 + v]);
+              xp[v] += xt[v];
+              yp[v] += kYRows ? 1 : tw;
+            }
+          }
+        }
+        continue;
+      }
+#pragma unroll
+      for (int m = 0; m < kSiSlots; ++m) {
+        if (32 * m >= n * ne) break;
+        const int o = off[m], u = o >> 16, r = (o >> 8) & 255, c = o & 255;
+        const int kl = max(0, min(kc, __shfl_sync(0xffffffffu, left, u)));  // 0 beyond the step
+        const bool tr = __shfl_sync(0xffffffffu, mj, u) < 0;
+        const int ku = (int)__reduce_max_sync(0xffffffffu, (unsigned)kl);
+        const double* xp = base + u * ss + (tr ? r : r * kl);
+        const double* yp = base + u * ss + sx + (kYRows ? c * kl : c);
+        const int xt = tr ? th : 1;
+        double v = acc[m];
+#pragma unroll 2
+        for (int tt = 0; tt < ku; ++tt, xp += xt, yp += kYRows ? 1 : tw)
+          if (tt < kl) v = fma(*xp, *yp, v);
+        acc[m] = v;
+      }
     }
   }
+  __syncwarp();
+#pragma unroll
+  for (int m = 0; m < kSiSlots; ++m)
+    if (lane + 32 * m < used) base[lane + 32 * m] = acc[m];
+  __syncwarp();
+  for (int e = lane; e < ne; e += 32) {
+    double v = used ? base[e] : 0.0;
+    for (int u = ne; u < used; u += ne) v += base[u + e];
+    base[e] = v;
+  }
+  __syncwarp();
 }
 
-// factor update: W(i,k) = A(i,k) + sigma [i = k] - sum_j W(i,j) L(k,j)^T over the block's term
-// list; warp gw serves item gw / split and the part gw % split of the list.  The term list
-// is walked in units of one term and 16 columns of t; the next unit's blocks are copied into
-// the warp's second stage buffer (cp.async) while the current unit is multiplied.
-__global__ void __launch_bounds__(kSiWarps * 32) si_update_kernel(SiDev s, const SiItem* __restrict__ items,
-                                                                   int64_t nitems, int split, int64_t E,
-                                                                   const double* __restrict__ A, double sigma) {
-  extern __shared__ double sh[];
+// factor update W(i,k) = A(i,k) + sigma [i = k] - sum_j W(i,j) L(k,j)^T and inversion, off-diagonal
+// blocks Z(i,k) = - sum_{j in struct(k)} Z(i,j) L(j,k).  parts = 0: a warp per item; else a CTA per
+// item and part, its warps sharing the part; with parts > 1 the parts go to P.
+template <int MODE>
+__global__ void __launch_bounds__(kSiWarps * 32, 4) si_sum_kernel(SiDev s, const SiItem* __restrict__ items,
+                                                                  int64_t nitems, int parts, int64_t E,
+                                                                  const double* __restrict__ A, double sigma) {
+  extern __shared__ __align__(16) double sh[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  if (gw >= nitems * split) return;
-  const int64_t itn = gw / split;
-  const int part = (int)(gw - itn * split);
+  const int64_t itn = parts ? (int64_t)(blockIdx.x / (unsigned)parts) : (int64_t)blockIdx.x * kSiWarps + w;
+  if (itn >= nitems) return;  // (only whole warps of parts = 0)
+  const int part = parts ? (int)(blockIdx.x % (unsigned)parts) : 0;
   const SiItem it = items[itn];
   const int i = s.colrow[it.blk], k = it.col;
   const int bi = s.bs[i], bk = s.bs[k];
-  const int ne = bi * bk;
-  const size_t half = (size_t)2 * s.maxb * kSiUp;       // one stage buffer: operand a | operand b
-  double* buf = sh + (size_t)w * 2 * half;
-  int rr[kSiEnt], cc[kSiEnt];
-  si_entries(it.e0, ne, bk, lane, rr, cc);
-  double acc[kSiEnt];
-  const int64_t ao = s.aoff[it.blk];
-#pragma unroll
-  for (int m = 0; m < kSiEnt; ++m) {
-    double v = 0.0;
-    if (part == 0 && rr[m] >= 0) {
-      if (ao >= 0) v = A[ao + it.e0 + lane + 32 * m];
-      if (i == k && rr[m] == cc[m]) v += sigma;
+  const int th = min(kTile, bi - it.r0), tw = min(kTile, bk - it.c0), ne = th * tw;
+  const int64_t* ptr = MODE == kSiUpdate ? s.uptr : s.optr;
+  const int64_t t0 = ptr[it.blk], nt = ptr[it.blk + 1] - t0;
+  const int64_t ways = parts ? (int64_t)parts * kSiWarps : 1, me = parts ? (int64_t)part * kSiWarps + w : 0;
+  si_sum<MODE>(s, t0 + nt * me / ways, t0 + nt * (me + 1) / ways, 0, bi, bk, it.r0, it.c0, th, tw,
+               sh + (size_t)w * kSiBuf, lane);
+  double* out = parts > 1 ? s.P + (int64_t)part * E + s.lpo[it.blk]
+                          : (MODE == kSiUpdate ? s.W : s.Z) + s.loff[it.blk];
+  const int64_t ao = MODE == kSiUpdate && part == 0 ? s.aoff[it.blk] : -1;
+  if (parts) __syncthreads();
+  for (int e = parts ? threadIdx.x : lane; e < ne; e += parts ? kSiWarps * 32 : 32) {
+    double v = sh[(parts ? 0 : (size_t)w * kSiBuf) + e];
+    if (parts)
+      for (int u = 1; u < kSiWarps; ++u) v += sh[(size_t)u * kSiBuf + e];
+    const int r = it.r0 + e / tw, c = it.c0 + e % tw;
+    double b = 0.0;
+    if (MODE == kSiUpdate && part == 0) {
+      if (ao >= 0) b = A[ao + (int64_t)r * bk + c];
+      if (i == k && r == c) b += sigma;
     }
-    acc[m] = v;
+    out[(int64_t)r * bk + c] = b - v;
   }
-  const int64_t t0 = s.uptr[it.blk], nt = s.uptr[it.blk + 1] - t0;
-  int64_t t = t0 + nt * part / split;
-  const int64_t te = t0 + nt * (part + 1) / split;
-  auto issue = [&](int64_t tt, int u0, double* dst) {
-    const int bw = s.uw[tt], bl = s.ul[tt];
-    const int bj = s.bs[s.colcol[bw]];
-    const int uw = min(kSiU, bj - u0), uw4 = (uw + 3) & ~3;
-    si_stage_async(dst, s.W + s.loff[bw] + u0, bi, uw, uw4, bj, 1, lane);             // W(i,j)
-    si_stage_async(dst + s.maxb * kSiUp, s.L + s.loff[bl] + u0, bk, uw, uw4, bj, 1, lane);  // L(k,j)
-  };
-  int u0 = 0, cur = 0;
-  if (t < te) issue(t, 0, buf);
-  si_cp_commit();
-  while (t < te) {
-    const int bj = s.bs[s.colcol[s.uw[t]]];
-    const int uwc = min(kSiU, bj - u0);
-    int64_t tn = t;
-    int un = u0 + kSiU;
-    if (un >= bj) {
-      tn = t + 1;
-      un = 0;
-    }
-    if (tn < te) issue(tn, un, buf + (cur ^ 1) * half);
-    si_cp_commit();
-    si_cp_wait1();
-    __syncwarp();
-    const double* cb = buf + cur * half;
-    si_dot(cb, cb + s.maxb * kSiUp, uwc, rr, cc, -1.0, acc);
-    __syncwarp();
-    t = tn;
-    u0 = un;
-    cur ^= 1;
-  }
-  si_cp_wait0();
-  double* out = split > 1 ? s.P + (int64_t)part * E + s.lpo[it.blk] : s.W + s.loff[it.blk];
-#pragma unroll
-  for (int m = 0; m < kSiEnt; ++m)
-    if (rr[m] >= 0) out[it.e0 + lane + 32 * m] = acc[m];
 }
 
-// Gauss-Jordan inverse of the bk x bk block M (row-major, shared) without pivoting; returns
-// false (in every thread) if a pivot was not a positive finite number.
-__device__ bool si_gauss_jordan(double* M, int bk, double* prow, double* pcol) {
-  bool ok = true;
-  for (int p = 0; p < bk; ++p) {
-    const double piv = M[p * bk + p];
-    if (!(piv > 0.0) || !isfinite(piv)) ok = false;
-    const double inv = 1.0 / piv;
-    for (int t = threadIdx.x; t < bk; t += blockDim.x) {
-      prow[t] = t == p ? inv : M[p * bk + t] * inv;
-      pcol[t] = M[t * bk + p];
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < bk * bk; idx += blockDim.x) {
-      const int r = idx / bk, c = idx - r * bk;
-      if (r == p) M[idx] = prow[c];
-      else M[idx] = (c == p ? 0.0 : M[idx]) - pcol[r] * prow[c];
-    }
-    __syncthreads();
-  }
-  return ok;
-}
-
-// Entry `idx` of CSC block q after the update of its level: W itself, or the sum of the
-// `split` parts in part order.
-__device__ __forceinline__ double si_assembled(const SiDev& s, const double* base, int64_t q, int idx, int split,
+// Entry idx behind block q's first of the level's sums: W or Z itself, or the parts added in order.
+__device__ __forceinline__ double si_assembled(const SiDev& s, const double* base, int64_t q, int64_t idx, int parts,
                                                int64_t E) {
-  if (split <= 1) return base[s.loff[q] + idx];
+  if (parts <= 1) return base[s.loff[q] + idx];
   const double* p = s.P + s.lpo[q] + idx;
   double v = p[0];
-  for (int t = 1; t < split; ++t) v += p[(int64_t)t * E];
+#pragma unroll 8
+  for (int t = 1; t < parts; ++t) v += p[(int64_t)t * E];
   return v;
 }
 
-// pivot: D(k,k)^{-1} and L(i,k) = W(i,k) D(k,k)^{-1}; CTA (x, y) serves supernode sn[x] and
-// the column blocks y*kSiSlice+1 .. of it; slice 0 stores D^{-1}.  With split > 1 the blocks
-// are first assembled from the update's parts (and W(i,k) stored).
-__global__ void __launch_bounds__(kSiThreads) si_pivot_kernel(SiDev s, const int32_t* __restrict__ sn, int split,
-                                                              int64_t E) {
-  extern __shared__ double smem[];
-  __shared__ double prow[kSiMaxB], pcol[kSiMaxB];
+// pivot: D(k,k)^{-1} by Gauss-Jordan without pivoting, then L(i,k) = W(i,k) D(k,k)^{-1}.  A column's
+// blocks lie one after the other with the same row pitch, so they are one tall matrix: CTA (x, y)
+// serves supernode sn[x] and the rows y * rows .. of it below the diagonal block; y = 0 stores
+// D^{-1}.  With parts > 1 the blocks are first assembled from the update's parts (and W(i,k)
+// stored).  Each CTA inverts D for itself; an entry of D stays in one thread's register, a pivot
+// step is one barrier and one division.
+__global__ void __launch_bounds__(kSiThreads) si_pivot_kernel(SiDev s, const int32_t* __restrict__ sn, int parts,
+                                                              int64_t E, int rows) {
+  extern __shared__ __align__(16) double sh[];  // D^{-1}, then a chunk of W
+  __shared__ double prow[2][kSiMaxB], pcol[2][kSiMaxB];
   const int k = sn[blockIdx.x];
-  const int bk = s.bs[k];
+  const int bk = s.bs[k], n2 = bk * bk, tid = threadIdx.x;
   const int64_t c0 = s.colptr[k], c1 = s.colptr[k + 1];
-  const int64_t q0 = c0 + 1 + (int64_t)blockIdx.y * kSiSlice;
-  if (blockIdx.y > 0 && q0 >= c1) return;
-  double* M = smem;
-  double* Wb = smem + (size_t)s.maxb * s.maxb;
-  for (int idx = threadIdx.x; idx < bk * bk; idx += blockDim.x) M[idx] = si_assembled(s, s.W, c0, idx, split, E);
-  __syncthreads();
-  const bool ok = si_gauss_jordan(M, bk, prow, pcol);
-  if (blockIdx.y == 0) {
-    if (!ok && threadIdx.x == 0) {
-      *(volatile unsigned int*)s.flag = 1u;
-      __threadfence_system();
-    }
-    double* Dinv = s.L + s.loff[c0];
-    for (int idx = threadIdx.x; idx < bk * bk; idx += blockDim.x) Dinv[idx] = M[idx];
+  const int64_t first = s.loff[c0] + n2, total = c1 > c0 + 1 ? s.loff[c1] - first : 0;  // entries below the diagonal
+  const int64_t e0 = (int64_t)blockIdx.y * rows * bk, e1 = min(total, e0 + (int64_t)rows * bk);
+  if (blockIdx.y > 0 && e0 >= total) return;
+  double v[kSiMaxB * kSiMaxB / kSiThreads];
+#pragma unroll
+  for (int m = 0; m < kSiMaxB * kSiMaxB / kSiThreads; ++m) {
+    if (m * kSiThreads >= n2) break;
+    const int idx = tid + m * kSiThreads;
+    if (idx < n2) v[m] = si_assembled(s, s.W, c0, idx, parts, E);
   }
-  const int64_t q1 = min(c1, q0 + kSiSlice);
-  for (int64_t q = q0; q < q1; ++q) {
-    const int bi = s.bs[s.colrow[q]];
-    double* Wq = s.W + s.loff[q];
-    for (int idx = threadIdx.x; idx < bi * bk; idx += blockDim.x) {
-      const double v = si_assembled(s, s.W, q, idx, split, E);
-      Wb[idx] = v;
-      if (split > 1) Wq[idx] = v;
+  bool ok = true;
+  for (int p = 0; p < bk; ++p) {
+    double* pr = prow[p & 1];
+    double* pc = pcol[p & 1];
+#pragma unroll
+    for (int m = 0; m < kSiMaxB * kSiMaxB / kSiThreads; ++m) {
+      if (m * kSiThreads >= n2) break;
+      const int idx = tid + m * kSiThreads;
+      if (idx < n2) {
+        const int r = idx / bk, c = idx - r * bk;
+        if (r == p) pr[c] = v[m];
+        if (c == p) pc[r] = v[m];
+      }
+    }
+    __syncthreads();  // the buffers of step p are rewritten at p + 2, behind the barrier of p + 1
+    const double piv = pr[p];
+    if (!(piv > 0.0) || !isfinite(piv)) ok = false;
+    const double inv = 1.0 / piv;
+#pragma unroll
+    for (int m = 0; m < kSiMaxB * kSiMaxB / kSiThreads; ++m) {
+      if (m * kSiThreads >= n2) break;
+      const int idx = tid + m * kSiThreads;
+      if (idx < n2) {
+        const int r = idx / bk, c = idx - r * bk;
+        const double q = c == p ? inv : pr[c] * inv;
+        v[m] = r == p ? q : (c == p ? 0.0 : v[m]) - pc[r] * q;
+      }
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < kSiMaxB * kSiMaxB / kSiThreads; ++m) {
+    if (m * kSiThreads >= n2) break;
+    const int idx = tid + m * kSiThreads;
+    if (idx < n2) {
+      sh[idx] = v[m];
+      if (blockIdx.y == 0) s.L[s.loff[c0] + idx] = v[m];
+    }
+  }
+  if (blockIdx.y == 0 && !ok && tid == 0) {
+    *(volatile unsigned int*)s.flag = 1u;
+    __threadfence_system();
+  }
+  double* Wb = sh + n2;
+  const int64_t step = kSiChunk / bk * bk;  // whole rows
+  for (int64_t e = e0; e < e1; e += step) {
+    const int len = (int)min(step, e1 - e);
+    __syncthreads();
+    for (int idx = tid; idx < len; idx += kSiThreads) {
+      const double w = si_assembled(s, s.W, c0, n2 + e + idx, parts, E);
+      Wb[idx] = w;
+      if (parts > 1) s.W[first + e + idx] = w;
     }
     __syncthreads();
-    double* Lq = s.L + s.loff[q];
-    for (int idx = threadIdx.x; idx < bi * bk; idx += blockDim.x) {
+    for (int idx = tid; idx < len; idx += kSiThreads) {
       const int r = idx / bk, c = idx - r * bk;
       const double* wr = Wb + r * bk;
       double t = 0.0;
-      for (int u = 0; u < bk; ++u) t = fma(wr[u], M[u * bk + c], t);
-      Lq[idx] = t;
+      for (int u = 0; u < bk; ++u) t = fma(wr[u], sh[u * bk + c], t);
+      s.L[first + e + idx] = t;
     }
-    __syncthreads();
   }
 }
 
-// inversion, off-diagonal blocks: Z(i,k) = - sum_{j in struct(k)} Z(i,j) L(j,k) over the block's
-// term list; warp gw serves item gw / split and the part gw % split of the list, staged and
-// prefetched as in the update.
-__global__ void __launch_bounds__(kSiWarps * 32) si_offdiag_kernel(SiDev s, const SiItem* __restrict__ items,
-                                                                    int64_t nitems, int split, int64_t E) {
-  extern __shared__ double sh[];
+// inversion, diagonal blocks: Z(k,k) = D^{-1} - sum_{j in struct(k)} Z(j,k)^T L(j,k).  A cluster of
+// CTAs (one, or kSiCluster where a column of the level is long) serves a supernode: each CTA
+// assembles its share of the Z(j,k) from the off-diagonal parts (parts > 1), its warps sum their
+// terms, and the CTAs' sums are added in order through distributed shared memory.
+__global__ void __launch_bounds__(kSiWarps * 32, 4) si_diag_kernel(SiDev s, const int32_t* __restrict__ sn, int parts,
+                                                                   int64_t E) {
+  extern __shared__ __align__(16) double sh[];
+  __shared__ double csum[kTile * kTile];
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int ctas = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  if (gw >= nitems * split) return;
-  const int64_t itn = gw / split;
-  const int part = (int)(gw - itn * split);
-  const SiItem it = items[itn];
-  const int i = s.colrow[it.blk], k = it.col;
-  const int bi = s.bs[i], bk = s.bs[k];
-  const int ne = bi * bk;
-  const size_t half = (size_t)2 * s.maxb * kSiUp;
-  double* buf = sh + (size_t)w * 2 * half;
-  int rr[kSiEnt], cc[kSiEnt];
-  si_entries(it.e0, ne, bk, lane, rr, cc);
-  double acc[kSiEnt];
-#pragma unroll
-  for (int m = 0; m < kSiEnt; ++m) acc[m] = 0.0;
-  const int64_t t0 = s.optr[it.blk], nt = s.optr[it.blk + 1] - t0;
-  int64_t t = t0 + nt * part / split;
-  const int64_t te = t0 + nt * (part + 1) / split;
-  auto issue = [&](int64_t tt, int u0, double* dst) {
-    const int zb = s.oz[tt], qq = s.ol[tt];
-    const int bj = s.bs[s.colrow[qq]];
-    const int uw = min(kSiU, bj - u0), uw4 = (uw + 3) & ~3;
-    if (zb < 0)  // Z(i,j) = Z(j,i)^T, block bj x bi
-      si_stage_async(dst, s.Z + s.loff[~zb] + (int64_t)u0 * bi, bi, uw, uw4, 1, bi, lane);
-    else
-      si_stage_async(dst, s.Z + s.loff[zb] + u0, bi, uw, uw4, bj, 1, lane);
-    si_stage_async(dst + s.maxb * kSiUp, s.L + s.loff[qq] + (int64_t)u0 * bk, bk, uw, uw4, 1, bk, lane);  // L(j,k)
-  };
-  int u0 = 0, cur = 0;
-  if (t < te) issue(t, 0, buf);
-  si_cp_commit();
-  while (t < te) {
-    const int bj = s.bs[s.colrow[s.ol[t]]];
-    const int uwc = min(kSiU, bj - u0);
-    int64_t tn = t;
-    int un = u0 + kSiU;
-    if (un >= bj) {
-      tn = t + 1;
-      un = 0;
-    }
-    if (tn < te) issue(tn, un, buf + (cur ^ 1) * half);
-    si_cp_commit();
-    si_cp_wait1();
-    __syncwarp();
-    const double* cb = buf + cur * half;
-    si_dot(cb, cb + s.maxb * kSiUp, uwc, rr, cc, -1.0, acc);
-    __syncwarp();
-    t = tn;
-    u0 = un;
-    cur ^= 1;
-  }
-  si_cp_wait0();
-  double* out = split > 1 ? s.P + (int64_t)part * E + s.lpo[it.blk] : s.Z + s.loff[it.blk];
-#pragma unroll
-  for (int m = 0; m < kSiEnt; ++m)
-    if (rr[m] >= 0) out[it.e0 + lane + 32 * m] = acc[m];
-}
-
-// inversion, diagonal blocks: Z(k,k) = D^{-1} - sum_{j in struct(k)} Z(j,k)^T L(j,k).  CTA
-// (x, y) serves supernode sn[x] and the column blocks y*kSiSlice+1 .. of it: with split > 1
-// it first assembles those Z(j,k) from the off-diagonal parts, then its warps split the
-// slice's terms and add them in warp order.  With one slice the CTA writes Z(k,k); with
-// several, each slice stores its sum in Q and the last slice to finish (counted per
-// supernode in `cnt`, which it resets) adds the slices in slice order and writes Z(k,k).
-__global__ void __launch_bounds__(kSiWarps * 32) si_diag_kernel(SiDev s, const int32_t* __restrict__ sn, int split,
-                                                                int64_t E, int slices, unsigned int* cnt,
-                                                                double* Q) {
-  extern __shared__ double sh[];
-  __shared__ int last;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int k = sn[blockIdx.x];
+  const int k = sn[blockIdx.x / (unsigned)ctas];
   const int bk = s.bs[k];
-  const int64_t c0 = s.colptr[k], c1 = s.colptr[k + 1];
-  const int64_t qs = c0 + 1 + (int64_t)blockIdx.y * kSiSlice, qe = min(c1, qs + kSiSlice);
-  if (split > 1 && qe > qs) {
-    const int64_t z0 = s.loff[qs], len = s.loff[qe] - z0;
-    const double* p = s.P + s.lpo[qs];
-    for (int64_t idx = threadIdx.x; idx < len; idx += blockDim.x) {
-      double v = p[idx];
-      for (int t = 1; t < split; ++t) v += p[(int64_t)t * E + idx];
-      s.Z[z0 + idx] = v;
-    }
+  const int64_t c0 = s.colptr[k] + 1, nt = s.colptr[k + 1] - c0;
+  const int64_t t0 = nt * rank / ctas, t1 = nt * (rank + 1) / ctas;  // this CTA's terms
+  if (parts > 1 && t1 > t0) {
+    const int64_t z0 = s.loff[c0 + t0], len = s.loff[c0 + t1] - z0;
+    for (int64_t idx = threadIdx.x; idx < len; idx += blockDim.x)
+      s.Z[z0 + idx] = si_assembled(s, s.Z, c0 + t0, idx, parts, E);
     __syncthreads();
   }
-  double* sa = sh + (size_t)w * 2 * s.maxb * kSiUp;
-  double* sb = sa + (size_t)s.maxb * kSiUp;
-  double* red = sh + (size_t)kSiWarps * 2 * s.maxb * kSiUp;  // [warp][kSiTileEnt]
-  const double* Dinv = s.L + s.loff[c0];
-  double* Zkk = s.Z + s.loff[c0];
-  const int ne = bk * bk;
-  const int64_t qst = (int64_t)s.maxb * s.maxb;                             // slice stride in Q
-  double* mine = Q + ((int64_t)blockIdx.x * slices + blockIdx.y) * qst;      // this slice's sum
-  for (int e0 = 0; e0 < ne; e0 += kSiTileEnt) {
-    int rr[kSiEnt], cc[kSiEnt];
-    si_entries(e0, ne, bk, lane, rr, cc);
-    double acc[kSiEnt];
-#pragma unroll
-    for (int m = 0; m < kSiEnt; ++m) acc[m] = 0.0;
-    for (int64_t q = qs + w; q < qe; q += kSiWarps) {
-      const int bj = s.bs[s.colrow[q]];
-      const double* Zq = s.Z + s.loff[q];  // bj x bk
-      const double* Lq = s.L + s.loff[q];
-      for (int u0 = 0; u0 < bj; u0 += kSiU) {
-        const int uw = min(kSiU, bj - u0), uw4 = (uw + 3) & ~3;
-        __syncwarp();
-        si_stage(sa, Zq + (int64_t)u0 * bk, bk, uw, uw4, 1, bk, lane);
-        si_stage(sb, Lq + (int64_t)u0 * bk, bk, uw, uw4, 1, bk, lane);
-        __syncwarp();
-        si_dot(sa, sb, uw, rr, cc, 1.0, acc);
+  const double* Dinv = s.L + s.loff[c0 - 1];
+  double* Zkk = s.Z + s.loff[c0 - 1];
+  for (int r0 = 0; r0 < bk; r0 += kTile)
+    for (int d0 = 0; d0 < bk; d0 += kTile) {
+      const int th = min(kTile, bk - r0), tw = min(kTile, bk - d0), ne = th * tw;
+      si_sum<kSiDiag>(s, t0 + (t1 - t0) * w / kSiWarps, t0 + (t1 - t0) * (w + 1) / kSiWarps, c0, bk, bk, r0, d0, th, tw,
+                      sh + (size_t)w * kSiBuf, lane);
+      __syncthreads();
+      for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+        double v = sh[e];
+        for (int u = 1; u < kSiWarps; ++u) v += sh[(size_t)u * kSiBuf + e];
+        csum[e] = v;
       }
+      cluster.sync();
+      for (int e = rank * kSiWarps * 32 + threadIdx.x; e < ne; e += ctas * kSiWarps * 32) {
+        double v = 0.0;
+        for (int u = 0; u < ctas; ++u) v += cluster.map_shared_rank(csum, u)[e];
+        const int at = (r0 + e / tw) * bk + d0 + e % tw;
+        Zkk[at] = Dinv[at] - v;
+      }
+      cluster.sync();  // no CTA reuses its sums or leaves while another reads them
     }
-#pragma unroll
-    for (int m = 0; m < kSiEnt; ++m) red[w * kSiTileEnt + lane + 32 * m] = acc[m];
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < kSiTileEnt && e0 + idx < ne; idx += blockDim.x) {
-      double v = red[idx];
-      for (int t = 1; t < kSiWarps; ++t) v += red[t * kSiTileEnt + idx];
-      if (slices == 1) Zkk[e0 + idx] = Dinv[e0 + idx] - v;
-      else mine[e0 + idx] = v;
-    }
-    __syncthreads();
-  }
-  if (slices == 1) return;
-  // the last slice of this supernode adds all slices in order
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(cnt + k, 1u) == (unsigned int)(slices - 1);
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  const double* all = Q + (int64_t)blockIdx.x * slices * qst;
-  for (int idx = threadIdx.x; idx < ne; idx += blockDim.x) {
-    double v = 0.0;
-    for (int t = 0; t < slices; ++t) v += ((volatile const double*)all)[(int64_t)t * qst + idx];
-    Zkk[idx] = Dinv[idx] - v;
-  }
-  if (threadIdx.x == 0) cnt[k] = 0u;
 }
 
 // out = alpha P_S(Z) + beta out: one warp per block of S
@@ -684,11 +633,10 @@ struct s_selinv_t {
   double flops_factor = 0.0, flops_invert = 0.0;
   // level lists (host offsets into the device arrays)
   std::vector<int64_t> upd_ptr, off_ptr, sn_ptr;
-  std::vector<int32_t> lvl_slices;  // pivot CTAs per supernode on each level
-  std::vector<int64_t> lvl_ent;     // entries of the blocks of each level's columns
-  std::vector<int32_t> upd_split, off_split;  // parts of the update and off-diagonal sums
-  unsigned int* cnt = nullptr;      // per supernode: slices of the diagonal kernel finished
-  double* Q = nullptr;              // slice sums of the diagonal kernel
+  std::vector<int32_t> lvl_rows, lvl_slices;  // rows of a pivot CTA, pivot CTAs per supernode
+  std::vector<int64_t> lvl_longest;           // longest struct(k) of each level
+  std::vector<int64_t> lvl_ent;               // entries of the blocks of each level's columns
+  std::vector<int32_t> upd_parts, off_parts;  // 0: a warp per item, else CTAs per item
   // device
   int32_t* bs = nullptr;
   int64_t* colptr = nullptr;
@@ -731,8 +679,6 @@ static void selinv_free(s_selinv_t* p) {
   cudaFree(p->aoff);
   cudaFree(p->lpo);
   cudaFree(p->P);
-  cudaFree(p->cnt);
-  cudaFree(p->Q);
   cudaFree(p->upd);
   cudaFree(p->off);
   cudaFree(p->sn);
@@ -764,7 +710,6 @@ static SiDev dev_of(const s_selinv_t* p) {
   s.Z = p->Z;
   s.P = p->P;
   s.flag = p->flag;
-  s.maxb = p->maxb;
   return s;
 }
 
@@ -911,45 +856,58 @@ static s_status selinv_build(s_selinv_t* p) {
   p->upd_ptr.assign(1, 0);
   p->off_ptr.assign(1, 0);
   p->sn_ptr.assign(1, 0);
+  p->lvl_rows.assign(H, 1);
   p->lvl_slices.assign(H, 1);
+  p->lvl_longest.assign(H, 0);
   p->lvl_ent.assign(H, 0);
-  p->upd_split.assign(H, 1);
-  p->off_split.assign(H, 1);
-  const int64_t target = 16LL * kSiWarps * sm_count();  // sixteen warps per SM sub-partition
-  int64_t scratch = 0, qneed = 0;
+  p->upd_parts.assign(H, 0);
+  p->off_parts.assign(H, 0);
+  const int64_t sms = sm_count();
+  int64_t scratch = 0;
   for (int32_t l = 0; l < H; ++l) {
-    int64_t longest = 0, ent = 0, maxu = 0, maxo = 0;
+    int64_t longest = 0, ent = 0, maxu = 0, maxo = 0, rows = 0, maxrows = 0;
     const int64_t u0 = (int64_t)upd.size(), o0 = (int64_t)off.size();
     for (int32_t k : bylvl[l]) {
       sn.push_back(k);
       longest = std::max<int64_t>(longest, colptr[k + 1] - colptr[k] - 1);
+      const int64_t below = (loff[colptr[k + 1]] - loff[colptr[k]]) / bs[k] - bs[k];
+      rows += below;
+      maxrows = std::max(maxrows, below);
       for (int64_t q = colptr[k]; q < colptr[k + 1]; ++q) {
         maxu = std::max<int64_t>(maxu, uptr[q + 1] - uptr[q]);
         maxo = std::max<int64_t>(maxo, optr[q + 1] - optr[q]);
-        const int ne = bs[colrow[q]] * bs[k];
+        const int bi = bs[colrow[q]], bk = bs[k];
         lpo[q] = ent;
-        ent += ne;
-        for (int e0 = 0; e0 < ne; e0 += kSiTileEnt) {
-          upd.push_back(SiItem{(int32_t)q, k, e0});
-          if (q > colptr[k]) off.push_back(SiItem{(int32_t)q, k, e0});
-        }
+        ent += (int64_t)bi * bk;
+        for (int r0 = 0; r0 < bi; r0 += kTile)
+          for (int c0 = 0; c0 < bk; c0 += kTile) {
+            upd.push_back(SiItem{(int32_t)q, k, (int16_t)r0, (int16_t)c0});
+            if (q > colptr[k]) off.push_back(SiItem{(int32_t)q, k, (int16_t)r0, (int16_t)c0});
+          }
       }
     }
     const int64_t nu = (int64_t)upd.size() - u0, no = (int64_t)off.size() - o0;
-    auto choose = [&](int64_t items, int64_t terms) {  // parts of at least kSiPartTerms terms
-      int64_t sp = items > 0 ? (target + items - 1) / items : 1;
-      sp = std::min<int64_t>(sp, std::min<int64_t>(kSiMaxSplit, (terms + kSiPartTerms - 1) / kSiPartTerms));
-      while (sp > 1 && sp * ent > (int64_t)1 << 27) --sp;  // scratch at most 1 GiB
-      return (int32_t)std::max<int64_t>(1, sp);
+    // Ways of a level's sums.  A warp's terms take an SM sub-partition's FP64 pipe 1 us each (10 x 10
+    // x 10), so a sum is spread until a warp holds kSiStepTerms of them or twice the resident
+    // warps are at work; a warp per item only where the items alone fill the SMs.
+    auto choose = [&](int64_t items, int64_t terms) -> int32_t {
+      const int64_t slots = 2 * sms * 4;  // twice the resident CTAs
+      if (items >= slots * kSiWarps || terms <= kSiStepTerms) return 0;
+      int64_t q = std::min<int64_t>((slots + items - 1) / std::max<int64_t>(items, 1),
+                                    (terms + kSiWarps * kSiStepTerms - 1) / (kSiWarps * kSiStepTerms));
+      q = std::max<int64_t>(1, std::min<int64_t>(q, kSiMaxParts));
+      while (q > 1 && q * ent > (int64_t)1 << 27) --q;  // scratch at most 1 GiB
+      return (int32_t)q;
     };
-    p->upd_split[l] = choose(nu, maxu);
-    p->off_split[l] = choose(no, maxo);
-    const int32_t sp = std::max(p->upd_split[l], p->off_split[l]);
-    if (sp > 1) scratch = std::max<int64_t>(scratch, (int64_t)sp * ent);
+    p->upd_parts[l] = choose(nu, maxu);
+    p->off_parts[l] = choose(no, maxo);
+    const int32_t parts = std::max(p->upd_parts[l], p->off_parts[l]);
+    if (parts > 1) scratch = std::max<int64_t>(scratch, (int64_t)parts * ent);
     p->lvl_ent[l] = ent;
-    p->lvl_slices[l] = (int32_t)std::max<int64_t>(1, (longest + kSiSlice - 1) / kSiSlice);
-    if (p->lvl_slices[l] > 1)
-      qneed = std::max<int64_t>(qneed, (int64_t)bylvl[l].size() * p->lvl_slices[l] * p->maxb * p->maxb);
+    p->lvl_longest[l] = longest;
+    // pivot CTAs: 32 rows each while the level leaves SMs idle, up to 256
+    p->lvl_rows[l] = (int32_t)std::min<int64_t>(256, std::max<int64_t>(32, (rows + sms * 4 - 1) / (sms * 4)));
+    p->lvl_slices[l] = (int32_t)std::max<int64_t>(1, (maxrows + p->lvl_rows[l] - 1) / p->lvl_rows[l]);
     p->upd_ptr.push_back((int64_t)upd.size());
     p->off_ptr.push_back((int64_t)off.size());
     p->sn_ptr.push_back((int64_t)sn.size());
@@ -968,9 +926,6 @@ static s_status selinv_build(s_selinv_t* p) {
   if (ce == cudaSuccess) ce = cudaMalloc(&p->L, vb);
   if (ce == cudaSuccess) ce = cudaMalloc(&p->Z, vb);
   if (ce == cudaSuccess && scratch > 0) ce = cudaMalloc(&p->P, sizeof(double) * (size_t)scratch);
-  if (ce == cudaSuccess && qneed > 0) ce = cudaMalloc(&p->Q, sizeof(double) * (size_t)qneed);
-  if (ce == cudaSuccess) ce = cudaMalloc(&p->cnt, sizeof(unsigned int) * (size_t)std::max(m, 1));
-  if (ce == cudaSuccess) ce = cudaMemset(p->cnt, 0, sizeof(unsigned int) * (size_t)std::max(m, 1));
   if (ce == cudaErrorMemoryAllocation) {
     cudaGetLastError();
     return set_error(S_ERR_NOMEM, "selected inversion: no device memory for the factor");
@@ -1046,18 +1001,12 @@ s_status s_selinv_stats(s_selinv p, int64_t* l_blocks, int64_t* l_entries, int32
   return S_OK;
 }
 
-// Dynamic shared memory of the block kernels (per-warp staging of two operand slices, and
-// the diagonal kernel's warp sums) and of the pivot kernel (D^{-1} and one W block).
-static size_t stage_bytes(const s_selinv_t* p) {  // two stage buffers per warp
-  return sizeof(double) * (size_t)kSiWarps * 4 * p->maxb * kSiUp;
-}
-static size_t diag_bytes(const s_selinv_t* p) {  // one stage buffer per warp and the warp sums
-  return sizeof(double) * ((size_t)kSiWarps * 2 * p->maxb * kSiUp + (size_t)kSiWarps * kSiTileEnt);
-}
-static size_t pivot_bytes(const s_selinv_t* p) { return sizeof(double) * 2 * (size_t)p->maxb * p->maxb; }
+// Dynamic shared memory of the sum kernels and of the pivot kernel (D^{-1} and a chunk of W).
+constexpr size_t kSiSumBytes = sizeof(double) * kSiWarps * kSiBuf;
+static size_t pivot_bytes(const s_selinv_t* p) { return sizeof(double) * ((size_t)p->maxb * p->maxb + kSiChunk); }
 
 static s_status set_smem(const void* fn, size_t bytes) {
-  if (bytes > 48 * 1024) SF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  if (bytes > 40 * 1024) SF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
   return S_OK;
 }
 
@@ -1067,22 +1016,22 @@ s_status s_selinv_factor(s_selinv p, const double* A, double sigma, void* stream
   cudaStream_t cs = (cudaStream_t)stream;
   const SiDev s = dev_of(p);
   s_status st;
-  if ((st = set_smem((const void*)si_update_kernel, stage_bytes(p))) ||
+  if ((st = set_smem((const void*)si_sum_kernel<kSiUpdate>, kSiSumBytes)) ||
       (st = set_smem((const void*)si_pivot_kernel, pivot_bytes(p))))
     return st;
   for (int32_t l = 0; l < p->height; ++l) {
     const int64_t n = p->upd_ptr[l + 1] - p->upd_ptr[l];
-    const int split = p->upd_split[l];
+    const int parts = p->upd_parts[l];
     if (n > 0) {
-      const int64_t grid = (n * split + kSiWarps - 1) / kSiWarps;
-      si_update_kernel<<<(unsigned)grid, kSiWarps * 32, stage_bytes(p), cs>>>(s, p->upd + p->upd_ptr[l], n, split,
-                                                                              p->lvl_ent[l], A, sigma);
+      const int64_t grid = parts ? n * parts : (n + kSiWarps - 1) / kSiWarps;
+      si_sum_kernel<kSiUpdate><<<(unsigned)grid, kSiWarps * 32, kSiSumBytes, cs>>>(s, p->upd + p->upd_ptr[l], n, parts,
+                                                                                   p->lvl_ent[l], A, sigma);
     }
     const int64_t ns = p->sn_ptr[l + 1] - p->sn_ptr[l];
     if (ns > 0) {
       dim3 g((unsigned)ns, (unsigned)p->lvl_slices[l]);
-      si_pivot_kernel<<<g, kSiThreads, pivot_bytes(p), cs>>>(s, p->sn + p->sn_ptr[l], n > 0 ? split : 1,
-                                                             p->lvl_ent[l]);
+      si_pivot_kernel<<<g, kSiThreads, pivot_bytes(p), cs>>>(s, p->sn + p->sn_ptr[l], parts, p->lvl_ent[l],
+                                                             p->lvl_rows[l]);
     }
   }
   SF_CUDA(cudaGetLastError());
@@ -1095,23 +1044,36 @@ s_status s_selinv_invert(s_selinv p, double alpha, double beta, double* out, voi
   if (p->m > 0) {
     const SiDev s = dev_of(p);
     s_status st;
-    if ((st = set_smem((const void*)si_offdiag_kernel, stage_bytes(p))) ||
-        (st = set_smem((const void*)si_diag_kernel, diag_bytes(p))))
+    if ((st = set_smem((const void*)si_sum_kernel<kSiOff>, kSiSumBytes)) ||
+        (st = set_smem((const void*)si_diag_kernel, kSiSumBytes)))
       return st;
-    SF_CUDA(cudaMemsetAsync(p->cnt, 0, sizeof(unsigned int) * (size_t)p->m, cs));
     for (int32_t l = p->height - 1; l >= 0; --l) {
       const int64_t n = p->off_ptr[l + 1] - p->off_ptr[l];
-      const int split = n > 0 ? p->off_split[l] : 1;
+      const int parts = p->off_parts[l];
       if (n > 0) {
-        const int64_t grid = (n * split + kSiWarps - 1) / kSiWarps;
-        si_offdiag_kernel<<<(unsigned)grid, kSiWarps * 32, stage_bytes(p), cs>>>(s, p->off + p->off_ptr[l], n,
-                                                                                 split, p->lvl_ent[l]);
+        const int64_t grid = parts ? n * parts : (n + kSiWarps - 1) / kSiWarps;
+        si_sum_kernel<kSiOff><<<(unsigned)grid, kSiWarps * 32, kSiSumBytes, cs>>>(s, p->off + p->off_ptr[l], n, parts,
+                                                                                  p->lvl_ent[l], nullptr, 0.0);
       }
       const int64_t ns = p->sn_ptr[l + 1] - p->sn_ptr[l];
       if (ns > 0) {
-        dim3 g((unsigned)ns, (unsigned)p->lvl_slices[l]);
-        si_diag_kernel<<<g, kSiWarps * 32, diag_bytes(p), cs>>>(s, p->sn + p->sn_ptr[l], split, p->lvl_ent[l],
-                                                                p->lvl_slices[l], p->cnt, p->Q);
+        // as many CTAs to a cluster as hold kSiStepTerms terms a warp and fit the SMs together
+        unsigned ctas = 1;
+        while (ctas < kSiCluster && p->lvl_longest[l] > (int64_t)ctas * kSiWarps * kSiStepTerms &&
+               2 * ctas * ns <= (int64_t)sm_count() * 4)
+          ctas *= 2;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)ns * ctas);
+        cfg.blockDim = dim3(kSiWarps * 32);
+        cfg.dynamicSmemBytes = kSiSumBytes;
+        cfg.stream = cs;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = ctas;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        SF_CUDA(cudaLaunchKernelEx(&cfg, si_diag_kernel, s, (const int32_t*)(p->sn + p->sn_ptr[l]), parts, p->lvl_ent[l]));
       }
     }
   }
