@@ -164,11 +164,12 @@ __global__ void __launch_bounds__(256) eval_colfwt_kernel(Geo g, int64_t n, int6
 
 // In-place row transform of one level: rows slots(c) of U (ld w) <- Q_c^T rows.  A warp owns 32 VEC
 // columns of a cluster and holds all their inputs in registers (MAXM of them), so the outputs go
-// straight back; Q is staged once per CTA and read four outputs at a time.  HBM / L2-bound: one read
+// straight back; Q is staged once per CTA, which takes all columns of its cluster where they fit 8
+// warps, and read four outputs at a time.  HBM / L2-bound: one read
 // and one write of the rows it transforms.  Same order of the sums as before (same
 // bits); N = 40000 on the sphere, all chunks and levels: 36.8 -> 26.3 ms.
 template <int MAXM, int VEC>
-__global__ void __launch_bounds__(128) rowfwt_reg_kernel(Geo g, const int32_t* __restrict__ lvl, int w,
+__global__ void __launch_bounds__(256) rowfwt_reg_kernel(Geo g, const int32_t* __restrict__ lvl, int w,
                                                          float* __restrict__ U) {
   __shared__ __align__(16) float Qs[MAXM * MAXM];
   __shared__ int ss[MAXM];
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(128) rowfwt_reg_kernel(Geo g, const int32_t* _
   }
   for (int e = threadIdx.x; e < m; e += blockDim.x) ss[e] = sl[e];
   __syncthreads();
-  const int j0 = ((int)blockIdx.y * 4 + (int)(threadIdx.x >> 5)) * 32 * VEC + (int)(threadIdx.x & 31);
+  const int j0 = ((int)(blockIdx.y * blockDim.x + threadIdx.x) >> 5) * 32 * VEC + (int)(threadIdx.x & 31);
   if (j0 - (int)(threadIdx.x & 31) >= w) return;
   float in[MAXM][VEC];
 #pragma unroll
@@ -623,8 +624,12 @@ static s_status values_impl(s_build b, double nu, double ell, double kscale, dou
       const int cnt = lvl_off[L + 1] - lvl_off[L];
       if (!cnt) continue;
       const int32_t* lv = dlvl + lvl_off[L];
-      if (lvl_m[L] <= 20) rowfwt_reg_kernel<20, 4><<<dim3(cnt, (w + 511) / 512), 128>>>(g, lv, w, dU);
-      else if (lvl_m[L] <= 40) rowfwt_reg_kernel<40, 2><<<dim3(cnt, (w + 255) / 256), 128>>>(g, lv, w, dU);
+      // a CTA per cluster with a warp per 128 (64) columns, the registers for the level's widest cluster
+      const int warps = (w + 127) / 128, warps2 = std::min(8, (w + 63) / 64);
+      if (lvl_m[L] <= 12) rowfwt_reg_kernel<12, 4><<<cnt, 32 * warps>>>(g, lv, w, dU);
+      else if (lvl_m[L] <= 20) rowfwt_reg_kernel<20, 4><<<cnt, 32 * warps>>>(g, lv, w, dU);
+      else if (lvl_m[L] <= 40)
+        rowfwt_reg_kernel<40, 2><<<dim3(cnt, (w + 64 * warps2 - 1) / (64 * warps2)), 32 * warps2>>>(g, lv, w, dU);
       else rowfwt_kernel<<<dim3(cnt, (w + kColTile - 1) / kColTile), 256>>>(g, lv, w, dU);
     }
     SF_CUDA(cudaGetLastError());
