@@ -237,6 +237,35 @@ __device__ __forceinline__ void d64_stage(uint32_t dst, const double* src, int r
   }
 }
 
+// Programmatic dependent launch, for chains of short kernels (a dependent launch costs about 2 us
+// between the kernels, and each kernel starts with a chain of loads of plan data).  A kernel
+// launched by launch_overlapped may start once every CTA of the stream's previous kernel has called
+// let_next_start() or left; it may read plan data at once, but must call wait_for_previous() (in
+// thread blocks that do work, and in at least one) before it reads or writes anything an earlier
+// kernel of the stream touches.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
+// `cluster` CTAs to a cluster (0: none).
+template <class... Par, class... Arg>
+cudaError_t launch_overlapped(void (*kern)(Par...), dim3 grid, int threads, size_t smem, unsigned cluster,
+                              cudaStream_t st, Arg... args) {
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 0 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<Par>(args)...);
+}
+
 }  // namespace sf
 
 struct s_plan_t {

@@ -34,9 +34,13 @@
 // on scheduling.  What bounds a level is its chain of latencies (term list, operand offsets, copies,
 // at least 8 terms' FP64 instructions) more than its operations; see the kernels.
 //
+// The launches overlap: each kernel starts while the one before it drains and fetches its first term
+// lists and offsets (plan data) before it waits for that one's results.  At N = 8192 in the plane
+// a factorization and an inversion are 1288 launches: 56.3 -> 53.9 ms.
+//
 // Every entry a launch reads was written by an earlier launch (descendants sit on lower
 // levels, ancestors on higher ones) or by its own CTA before a barrier, so the kernels need
-// no synchronisation beyond stream order and no waits.
+// no synchronisation beyond that.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -147,6 +151,7 @@ __device__ __forceinline__ void si_sum(const SiDev& s, int64_t t, int64_t te, in
   };
   const double* xall = MODE == kSiUpdate ? s.W : s.Z;
   fetch(t);
+  wait_for_previous();
   for (; t < te; t += S) {
     const int n = (int)min((int64_t)S, te - t);
     const int mj = nj;
@@ -237,8 +242,9 @@ __device__ __forceinline__ void si_sum(const SiDev& s, int64_t t, int64_t te, in
 template <int MODE>
 __global__ void __launch_bounds__(kSiWarps * 32, 4) si_sum_kernel(SiDev s, const SiItem* __restrict__ items,
                                                                   int64_t nitems, int parts, int64_t E,
-                                                                  const double* __restrict__ A, double sigma) {
+                                                                  const double* A, double sigma) {
   extern __shared__ __align__(16) double sh[];
+  let_next_start();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t itn = parts ? (int64_t)(blockIdx.x / (unsigned)parts) : (int64_t)blockIdx.x * kSiWarps + w;
   if (itn >= nitems) return;  // (only whole warps of parts = 0)
@@ -296,7 +302,9 @@ __global__ void __launch_bounds__(kSiThreads) si_pivot_kernel(SiDev s, const int
   const int64_t c0 = s.colptr[k], c1 = s.colptr[k + 1];
   const int64_t first = s.loff[c0] + n2, total = c1 > c0 + 1 ? s.loff[c1] - first : 0;  // entries below the diagonal
   const int64_t e0 = (int64_t)blockIdx.y * rows * bk, e1 = min(total, e0 + (int64_t)rows * bk);
+  let_next_start();
   if (blockIdx.y > 0 && e0 >= total) return;
+  wait_for_previous();
   double v[kSiMaxB * kSiMaxB / kSiThreads];
 #pragma unroll
   for (int m = 0; m < kSiMaxB * kSiMaxB / kSiThreads; ++m) {
@@ -383,6 +391,8 @@ __global__ void __launch_bounds__(kSiWarps * 32, 4) si_diag_kernel(SiDev s, cons
   const int bk = s.bs[k];
   const int64_t c0 = s.colptr[k] + 1, nt = s.colptr[k + 1] - c0;
   const int64_t t0 = nt * rank / ctas, t1 = nt * (rank + 1) / ctas;  // this CTA's terms
+  let_next_start();
+  wait_for_previous();
   if (parts > 1 && t1 > t0) {
     const int64_t z0 = s.loff[c0 + t0], len = s.loff[c0 + t1] - z0;
     for (int64_t idx = threadIdx.x; idx < len; idx += blockDim.x)
@@ -1024,14 +1034,14 @@ s_status s_selinv_factor(s_selinv p, const double* A, double sigma, void* stream
     const int parts = p->upd_parts[l];
     if (n > 0) {
       const int64_t grid = parts ? n * parts : (n + kSiWarps - 1) / kSiWarps;
-      si_sum_kernel<kSiUpdate><<<(unsigned)grid, kSiWarps * 32, kSiSumBytes, cs>>>(s, p->upd + p->upd_ptr[l], n, parts,
-                                                                                   p->lvl_ent[l], A, sigma);
+      SF_CUDA(launch_overlapped(si_sum_kernel<kSiUpdate>, dim3((unsigned)grid), kSiWarps * 32, kSiSumBytes, 0, cs, s,
+                        p->upd + p->upd_ptr[l], n, parts, p->lvl_ent[l], A, sigma));
     }
     const int64_t ns = p->sn_ptr[l + 1] - p->sn_ptr[l];
     if (ns > 0) {
       dim3 g((unsigned)ns, (unsigned)p->lvl_slices[l]);
-      si_pivot_kernel<<<g, kSiThreads, pivot_bytes(p), cs>>>(s, p->sn + p->sn_ptr[l], parts, p->lvl_ent[l],
-                                                             p->lvl_rows[l]);
+      SF_CUDA(launch_overlapped(si_pivot_kernel, g, kSiThreads, pivot_bytes(p), 0, cs, s, p->sn + p->sn_ptr[l], parts,
+                        p->lvl_ent[l], p->lvl_rows[l]));
     }
   }
   SF_CUDA(cudaGetLastError());
@@ -1052,8 +1062,8 @@ s_status s_selinv_invert(s_selinv p, double alpha, double beta, double* out, voi
       const int parts = p->off_parts[l];
       if (n > 0) {
         const int64_t grid = parts ? n * parts : (n + kSiWarps - 1) / kSiWarps;
-        si_sum_kernel<kSiOff><<<(unsigned)grid, kSiWarps * 32, kSiSumBytes, cs>>>(s, p->off + p->off_ptr[l], n, parts,
-                                                                                  p->lvl_ent[l], nullptr, 0.0);
+        SF_CUDA(launch_overlapped(si_sum_kernel<kSiOff>, dim3((unsigned)grid), kSiWarps * 32, kSiSumBytes, 0, cs, s,
+                          p->off + p->off_ptr[l], n, parts, p->lvl_ent[l], (const double*)nullptr, 0.0));
       }
       const int64_t ns = p->sn_ptr[l + 1] - p->sn_ptr[l];
       if (ns > 0) {
@@ -1062,18 +1072,8 @@ s_status s_selinv_invert(s_selinv p, double alpha, double beta, double* out, voi
         while (ctas < kSiCluster && p->lvl_longest[l] > (int64_t)ctas * kSiWarps * kSiStepTerms &&
                2 * ctas * ns <= (int64_t)sm_count() * 4)
           ctas *= 2;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)ns * ctas);
-        cfg.blockDim = dim3(kSiWarps * 32);
-        cfg.dynamicSmemBytes = kSiSumBytes;
-        cfg.stream = cs;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = ctas;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        SF_CUDA(cudaLaunchKernelEx(&cfg, si_diag_kernel, s, (const int32_t*)(p->sn + p->sn_ptr[l]), parts, p->lvl_ent[l]));
+        SF_CUDA(launch_overlapped(si_diag_kernel, dim3((unsigned)ns * ctas), kSiWarps * 32, kSiSumBytes, ctas, cs, s,
+                          p->sn + p->sn_ptr[l], parts, p->lvl_ent[l]));
       }
     }
   }
