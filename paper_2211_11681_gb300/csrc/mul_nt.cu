@@ -37,19 +37,21 @@
 // (a bulk copy issues from uniform registers, so a warp sends its 16 copies one lane at a time):
 // 41.5 against 37.6 ms for the three products of a gradient step at N = 6000 in space, q = 2.
 //
-// Sums: even and odd t are two float partials per entry; after the first step, then every 8 (16 of
-// 8 blocks at once), they are added and folded into the running sum with an error-free two-sum,
+// Sums: even and odd t are two float partials per entry; after the first step, then every 4 (8 of
+// wide tiles), they are added and folded into the running sum with an error-free two-sum,
 // the rounding error carried in the partial.  The lists run from coarse to fine clusters, so
 // the first step holds the largest terms: folded at once, it no longer makes the small terms
 // that follow round at its size.  At the end the groups' sums are combined the same way in
 // group order.  The order is fixed (deterministic).  Error against 64 bits, geometric mean over 8
-// matrices of 500 to 9900 points: 0.6e-7 to 1.4e-7 in the four families with 20- and 10-wide
-// blocks (1.1e-7 to 4.0e-7 with the replaced kernel's folds every 4 lambda blocks).
+// matrices of 500 to 9900 points: 0.4e-7 to 1.4e-7 in the four families with 20- and 10-wide
+// blocks (1.1e-7 to 4.0e-7 with the replaced kernel's folds every 4 lambda blocks).  Narrow tiles
+// folded only every 16 steps were 0.8 % faster, but left the float square root at N = 2000 in space,
+// whose factors are near the identity, 2.6e-7 off (1.1e-7 now, 2.0e-7 with the replaced kernel).
 //
 // Measured against the kernel this replaces (K-major slices, in-kernel intersection, one half-warp
-// per lambda block): N = 50000 in the plane, 10-wide blocks, B not symmetric 9.27 -> 4.07 ms; N = 65536 in
-// space, 20-wide blocks, B = A symmetric 39.1 -> 30.5 ms (37.6 TFLOP/s); N = 1000 in the plane
-// 192 -> 82 us; three products of a gradient step, N = 6000, 10-wide blocks 107.6 -> 36.8 ms.
+// per lambda block): N = 50000 in the plane, 10-wide blocks, B not symmetric 9.27 -> 3.90 ms; N = 65536 in
+// space, 20-wide blocks, B = A symmetric 39.1 -> 30.4 ms (37.7 TFLOP/s); N = 1000 in the plane
+// 192 -> 82 us; three products of a gradient step, N = 6000, 10-wide blocks 107.6 -> 35.4 ms.
 #include <algorithm>
 #include <cstring>
 
@@ -174,7 +176,7 @@ __global__ void nt_tile_kernel(int64_t nb, const int32_t* __restrict__ bsize, co
 }
 
 // 16-byte asynchronous copy global -> shared: through L1 for the narrow tiles (GL = 4), whose
-// neighbours re-read the same small slices soon (gradient step at N = 6000 36.6 -> 34.9 ms), past
+// neighbours re-read the same small slices soon (gradient step at N = 6000 36.6 -> 34.9 ms before the folds every 4 steps), past
 // L1 for the others (with it N = 65536 in space took 35.4 instead of 30.4 ms).
 template <bool L1>
 __device__ __forceinline__ void nt_cp16(uint32_t dst, const float* src) {
@@ -224,7 +226,7 @@ __device__ __forceinline__ void nt_tile(const NtArgs& a, const NtTile& tile, flo
   constexpr int SLOT = kNtBuf / S, KMAX = S == 8 ? 10 : S == 4 ? 12 : kNtKC;
   // 16-byte pieces a lane copies of an X and of a Y slice of up to KMAX
   constexpr int CX = (GR * MR * KMAX / 4 + GL - 1) / GL, CY = (TW * KMAX / 4 + GL - 1) / GL;
-  constexpr int FOLD = S == 8 ? 16 : 8;  // steps per two-sum fold: partials of about 80 terms
+  constexpr int FOLD = S == 2 ? 8 : 4;  // steps per two-sum fold: partials of 20 to 80 terms
   static_assert(S * ((NE + 1) & ~1) * 2 <= 2 * kNtBuf, "the group sums reuse the stage buffers");
   static_assert((GR * MR + TW) * KMAX <= SLOT && (GR * MR + TW) * kNtKC <= (S == 2 ? 1 : 2) * SLOT, "slot too small");
   const int g = lane / GL, gl = lane % GL, mr = gl / GC, mc = gl % GC;
