@@ -47,11 +47,15 @@
 // blocks (1.1e-7 to 4.0e-7 with the replaced kernel's folds every 4 lambda blocks).  Narrow tiles
 // folded only every 16 steps were 0.8 % faster, but left the float square root at N = 2000 in space,
 // whose factors are near the identity, 2.6e-7 off (1.1e-7 now, 2.0e-7 with the replaced kernel).
+// Within a block t runs downwards, so a cluster's coarsest samplets, the largest terms of the
+// dominant entries, are added last and round once (they alone decide the error's norm on matrices
+// of a few thousand points: N = 5000 in the plane 6.8e-8 -> 1.7e-8 over 6 matrices, 1.4e-7 with the
+// replaced kernel); upwards was 0.4 % faster.
 //
 // Measured against the kernel this replaces (K-major slices, in-kernel intersection, one half-warp
-// per lambda block): N = 50000 in the plane, 10-wide blocks, B not symmetric 9.27 -> 3.90 ms; N = 65536 in
-// space, 20-wide blocks, B = A symmetric 39.1 -> 30.4 ms (37.7 TFLOP/s); N = 1000 in the plane
-// 192 -> 81 us; three products of a gradient step, N = 6000, 10-wide blocks 107.6 -> 35.4 ms.
+// per lambda block): N = 50000 in the plane, 10-wide blocks, B not symmetric 9.27 -> 4.0 ms; N = 65536 in
+// space, 20-wide blocks, B = A symmetric 39.1 -> 30.5 ms (37.6 TFLOP/s); N = 1000 in the plane
+// 192 -> 83 us; three products of a gradient step, N = 6000, 10-wide blocks 107.6 -> 35.6 ms.
 #include <algorithm>
 #include <cstring>
 
@@ -266,10 +270,13 @@ __device__ __forceinline__ void nt_tile(const NtArgs& a, const NtTile& tile, flo
     if (cn > 0) {
       asm volatile("cp.async.wait_group 1;\n" ::: "memory");
       __syncwarp();
-      const float* xs = wbase + cxs + mr * (2 * MR);
-      const float* ys = wbase + cys + mc * (2 * MC);
+      // downwards: a cluster's first samplets are its coarsest, their terms the largest
+      const float* xs = wbase + cxs + mr * (2 * MR) + ckc * th;
+      const float* ys = wbase + cys + mc * (2 * MC) + ckc * tw;
 #pragma unroll 2
-      for (int t = 0; t < ckc; t += 2, xs += 2 * th, ys += 2 * tw) {
+      for (int t = ckc; t > 0; t -= 2) {
+        xs -= 2 * th;
+        ys -= 2 * tw;
         unsigned long long xv[MR];
 #pragma unroll
         for (int i = 0; i < MR; ++i) xv[i] = reinterpret_cast<const unsigned long long*>(xs)[i];
