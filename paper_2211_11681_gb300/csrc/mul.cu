@@ -1955,7 +1955,12 @@ extern "C" s_status s_plan_set_symmetric_a(s_plan p, int symmetric) {
   if (symmetric) {
     // the pattern must be symmetric: CSR and CSC index lists coincide
     if (A->rowptr.size() < 2) return S_OK;
-    std::vector<int64_t> cnt(A->d.nc + 1, 0);
+    std::vector<int64_t> cnt;
+    try {
+      cnt.assign(A->d.nc + 1, 0);
+    } catch (const std::bad_alloc&) {
+      return set_error(S_ERR_NOMEM, "s_plan_set_symmetric_a: host allocation");
+    }
     for (int32_t c : A->colidx) cnt[c + 1]++;
     for (int32_t i = 0; i < A->d.nc; ++i)
       if (cnt[i + 1] != A->rowptr[i + 1] - A->rowptr[i])

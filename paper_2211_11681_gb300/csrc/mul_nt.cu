@@ -58,6 +58,7 @@
 // 192 -> 83 us; three products of a gradient step, N = 6000, 10-wide blocks 107.6 -> 35.6 ms.
 #include <algorithm>
 #include <cstring>
+#include <new>
 
 #include "common.cuh"
 
@@ -458,10 +459,8 @@ void nt_free_side(NtSideDesc* s) {
 
 // Configure one side of the packed product: `pat` is the stored operand's pattern, `list` the
 // row (X) or column (Y) lists of op(.), `trans` whether the packed slice is the transpose of
-// the stored block.  Where there is no memory for the packed copy the side stays unconfigured
-// (off = nullptr) and the product runs on the tile kernel, which reads the operands as stored.
+// the stored block.
 static s_status nt_side(const s_pattern_t* pat, const Side& list, bool trans, NtSideDesc* s) {
-  nt_free_side(s);
   s->ptr = list.ptr;
   s->idx = list.idx;
   s->blk = list.blk;
@@ -469,13 +468,7 @@ static s_status nt_side(const s_pattern_t* pat, const Side& list, bool trans, Nt
   s->trans = trans;
   s_status st = padded_offsets(pat, trans, &s->poff, &s->len);
   if (st) return st;
-  const cudaError_t e = cudaMalloc(&s->scratch, sizeof(float) * std::max<int64_t>(s->len, 1));
-  if (e == cudaErrorMemoryAllocation) {
-    cudaGetLastError();
-    s->scratch = nullptr;
-    return S_OK;
-  }
-  SF_CUDA(e);
+  SF_CUDA(cudaMalloc(&s->scratch, sizeof(float) * std::max<int64_t>(s->len, 1)));
   s->off = s->poff;
   return S_OK;
 }
@@ -494,14 +487,11 @@ void nt_free_lists(MulDesc* d) {
 
 // Counts the lists of a configured descriptor, lays out the ranges of blocks that go through the
 // workspace together (one range: the plan keeps the lists, which are written here) and
-// allocates.  Without memory for them the descriptor stays without lists and the product runs
-// on the tile kernel.  All work is on the default stream and finished on return.
+// allocates.  All work is on the default stream and finished on return.
 static s_status nt_build_lists(MulDesc* d) {
-  nt_free_lists(d);
   SF_CUDA(cudaFuncSetAttribute(mul_f32_nt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNtSmem));
   SF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d->nt_per_sm, mul_f32_nt_kernel, kNtWarps * 32, kNtSmem));
   d->nt_per_sm = std::max(d->nt_per_sm, 1);
-  if (!d->ntx.off || !d->nty.off) return S_OK;
   // the entries count operand offsets in 4 floats with 32 bits, t in 16
   if ((d->ntx.len >> 2) > (int64_t)UINT32_MAX || (d->nty.len >> 2) > (int64_t)UINT32_MAX) return S_OK;
   for (const s_pattern_t* q : {d->px, d->py})
@@ -509,18 +499,23 @@ static s_status nt_build_lists(MulDesc* d) {
   const s_pattern_t* C = d->pc;
   const int64_t nb = C->d.nblocks;
   std::vector<int64_t> eptr(nb + 1, 0), tptr(nb + 1, 0);
-  int32_t* cnt = nullptr;
-  cudaError_t e = cudaMalloc(&cnt, sizeof(int32_t) * std::max<int64_t>(nb, 1));
+  struct Temp {  // device memory of this call
+    void* p = nullptr;
+    ~Temp() { cudaFree(p); }
+  };
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((nb + 7) / 8, (int64_t)sm_count() * 64));
-  if (e == cudaSuccess && nb > 0) {
-    nt_list_kernel<false><<<grid, 256>>>(list_side(d->ntx), list_side(d->nty), C->d.bsize, C->d.brow, C->d.colidx, 0, nb,
-                                         cnt, nullptr, 0, nullptr);
-    e = cudaGetLastError();
+  {
+    Temp cnt;
     std::vector<int32_t> h(nb);
-    if (e == cudaSuccess) e = cudaMemcpy(h.data(), cnt, sizeof(int32_t) * nb, cudaMemcpyDeviceToHost);
+    SF_CUDA(cudaMalloc(&cnt.p, sizeof(int32_t) * std::max<int64_t>(nb, 1)));
+    if (nb > 0) {
+      nt_list_kernel<false><<<grid, 256>>>(list_side(d->ntx), list_side(d->nty), C->d.bsize, C->d.brow, C->d.colidx, 0, nb,
+                                           (int32_t*)cnt.p, nullptr, 0, nullptr);
+      SF_CUDA(cudaGetLastError());
+      SF_CUDA(cudaMemcpy(h.data(), cnt.p, sizeof(int32_t) * nb, cudaMemcpyDeviceToHost));
+    }
     for (int64_t k = 0; k < nb; ++k) eptr[k + 1] = eptr[k] + h[k];
   }
-  cudaFree(cnt);
   const int64_t most = kNtListMax / (int64_t)sizeof(NtEntry), work = kNtListWork / (int64_t)sizeof(NtEntry);
   int64_t room = 0;  // entries to allocate
   NtRange r{0, 0, 0, 0, 0};
@@ -538,30 +533,24 @@ static s_status nt_build_lists(MulDesc* d) {
   }
   if (nb > 0) d->nt_ranges.push_back(r);
   for (NtRange& q : d->nt_ranges) q.base = eptr[q.k0];
-  if (e == cudaSuccess) e = cudaMalloc(&d->nt_eptr, sizeof(int64_t) * (nb + 1));
-  if (e == cudaSuccess) e = cudaMemcpy(d->nt_eptr, eptr.data(), sizeof(int64_t) * (nb + 1), cudaMemcpyHostToDevice);
-  int64_t* dtptr = nullptr;
-  if (e == cudaSuccess) e = cudaMalloc(&dtptr, sizeof(int64_t) * (nb + 1));
-  if (e == cudaSuccess) e = cudaMemcpy(dtptr, tptr.data(), sizeof(int64_t) * (nb + 1), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&d->nt_tiles, sizeof(NtTile) * std::max<int64_t>(tptr[nb], 1));
-  if (e == cudaSuccess && nb > 0) {
-    nt_tile_kernel<<<(unsigned)((nb + 255) / 256), 256>>>(nb, C->d.bsize, C->d.brow, C->d.colidx, C->d.voff, dtptr,
-                                                          d->nt_eptr, d->nt_tiles);
-    e = cudaGetLastError();
+  SF_CUDA(cudaMalloc(&d->nt_eptr, sizeof(int64_t) * (nb + 1)));
+  SF_CUDA(cudaMemcpy(d->nt_eptr, eptr.data(), sizeof(int64_t) * (nb + 1), cudaMemcpyHostToDevice));
+  Temp dtptr;
+  SF_CUDA(cudaMalloc(&dtptr.p, sizeof(int64_t) * (nb + 1)));
+  SF_CUDA(cudaMemcpy(dtptr.p, tptr.data(), sizeof(int64_t) * (nb + 1), cudaMemcpyHostToDevice));
+  SF_CUDA(cudaMalloc(&d->nt_tiles, sizeof(NtTile) * std::max<int64_t>(tptr[nb], 1)));
+  if (nb > 0) {
+    nt_tile_kernel<<<(unsigned)((nb + 255) / 256), 256>>>(nb, C->d.bsize, C->d.brow, C->d.colidx, C->d.voff,
+                                                          (const int64_t*)dtptr.p, d->nt_eptr, d->nt_tiles);
+    SF_CUDA(cudaGetLastError());
   }
-  if (e == cudaSuccess) e = cudaMalloc(&d->nt_ent, sizeof(NtEntry) * std::max<int64_t>(room, 1));
-  if (e == cudaSuccess && d->nt_ranges.size() == 1) {
+  SF_CUDA(cudaMalloc(&d->nt_ent, sizeof(NtEntry) * std::max<int64_t>(room, 1)));
+  if (d->nt_ranges.size() == 1) {
     nt_list_kernel<true><<<grid, 256>>>(list_side(d->ntx), list_side(d->nty), C->d.bsize, C->d.brow, C->d.colidx, 0, nb,
                                         nullptr, d->nt_eptr, 0, d->nt_ent);
-    e = cudaGetLastError();
+    SF_CUDA(cudaGetLastError());
   }
-  if (e == cudaSuccess) e = cudaDeviceSynchronize();
-  cudaFree(dtptr);
-  if (e != cudaSuccess) {
-    nt_free_lists(d);
-    if (e != cudaErrorMemoryAllocation) return cuda_error(e, "packed float product: lists");
-    cudaGetLastError();
-  }
+  SF_CUDA(cudaDeviceSynchronize());
   return S_OK;
 }
 
@@ -572,7 +561,7 @@ static s_status nt_build_lists(MulDesc* d) {
 // CSR-row entry (nu', lambda) has a row per column of op(Y); with op(Y) = Y the CSC-column entry
 // (lambda, nu') is transposed, unless `y_sym` (Y = X declared symmetric and called with one
 // buffer) lets the kernel read Y(nu', lambda) through Y's own CSR rows.
-s_status nt_configure(MulDesc* d, bool x_trans, bool y_trans, bool y_sym) {
+static s_status nt_sides(MulDesc* d, bool x_trans, bool y_trans, bool y_sym) {
   const DevPattern& px = d->px->d;
   const DevPattern& py = d->py->d;
   Side xl = x_trans ? Side{px.colptr, px.rowidx, px.cscblk, px.voff, true}
@@ -588,21 +577,42 @@ s_status nt_configure(MulDesc* d, bool x_trans, bool y_trans, bool y_sym) {
     yl = Side{py.colptr, py.rowidx, py.cscblk, py.voff, true};
     ytrans = true;
   }
-  if (y_sym && !x_trans) {
-    // B = A read through A's rows: the same packed blocks as the X side, one copy for both
-    nt_free_side(&d->nty);
-    d->nty.ptr = yl.ptr;
-    d->nty.idx = yl.idx;
-    d->nty.blk = yl.blk;
-    d->nty.pat = d->py;
-    d->nty.off = d->ntx.off;
-    d->nty.len = d->ntx.len;
-    d->nty.from_x = true;
-  } else if ((st = nt_side(d->py, yl, ytrans, &d->nty))) {
-    return st;
-  }
+  if (!y_sym || x_trans) return nt_side(d->py, yl, ytrans, &d->nty);
+  // B = A read through A's rows: the same packed blocks as the X side, one copy for both
+  d->nty.ptr = yl.ptr;
+  d->nty.idx = yl.idx;
+  d->nty.blk = yl.blk;
+  d->nty.pat = d->py;
+  d->nty.off = d->ntx.off;
+  d->nty.len = d->ntx.len;
+  d->nty.from_x = true;
+  return S_OK;
+}
+
+// Configures a descriptor for the packed kernel, or leaves it without packed copies and lists, all of
+// them: the old ones go first, since lists say where blocks start in copies that are laid out
+// anew.  Where device or host memory runs out the descriptor stays without them and the product
+// runs on the tile kernel, which reads the operands as stored.
+s_status nt_configure(MulDesc* d, bool x_trans, bool y_trans, bool y_sym) {
+  nt_free_lists(d);
+  nt_free_side(&d->ntx);
+  nt_free_side(&d->nty);
   d->nt_ysym = y_sym;
-  return nt_build_lists(d);
+  s_status st;
+  try {
+    st = nt_sides(d, x_trans, y_trans, y_sym);
+    if (!st) st = nt_build_lists(d);
+  } catch (const std::bad_alloc&) {
+    st = S_ERR_NOMEM;
+  }
+  if (st || !d->nt_ent) {
+    nt_free_lists(d);
+    nt_free_side(&d->ntx);
+    nt_free_side(&d->nty);
+  }
+  if (st != S_ERR_NOMEM) return st;
+  cudaGetLastError();  // the failed allocation is dealt with
+  return S_OK;
 }
 
 static NtPack pack_of(const NtSideDesc& s, const void* src) {
@@ -611,7 +621,7 @@ static NtPack pack_of(const NtSideDesc& s, const void* src) {
 }
 
 bool nt_usable(const MulDesc& d, const void* X, const void* Y) {
-  if (!d.nt_ent) return false;
+  if (!d.nt_ent || !d.ntx.off || !d.nty.off) return false;
   // a symmetric Y side reads B through A's rows: only valid for B = A
   return !d.nt_ysym || X == Y;
 }

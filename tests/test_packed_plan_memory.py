@@ -1,0 +1,111 @@
+"""Host logic of the packed float product's plan (mul_nt.cu) when memory runs out: the library's
+object files linked with a CUDA runtime over host memory (fake_cuda_runtime.cpp), in which any
+device or host allocation can be made to fail.  No GPU: the launches are only counted and their
+operands checked against the live allocations."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+class Fake:
+    """The library over host memory, with the few calls the tests make."""
+
+    def __init__(self, path):
+        self.lib = L = ctypes.CDLL(path, mode=ctypes.RTLD_LOCAL)
+        for n in ("fake_used", "fake_bad", "fake_device_calls", "fake_host_calls", "fake_launches"):
+            getattr(L, n).restype = ctypes.c_int64
+        for n in ("fake_pool", "fake_fail_device", "fake_fail_host"):
+            getattr(L, n).argtypes = [ctypes.c_int64]
+        L.s_pattern_nnz.restype = ctypes.c_int64
+        for n in ("s_pattern_nnz", "s_pattern_destroy", "s_plan_destroy"):
+            getattr(L, n).argtypes = [ctypes.c_void_p]
+        L.s_plan_set_symmetric_a.argtypes = [ctypes.c_void_p, ctypes.c_int]
+
+    def pattern(self, sizes):
+        nc = len(sizes)
+        bo = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+        rp, ci = (np.arange(nc + 1) * nc).astype(np.int64), np.tile(np.arange(nc), nc).astype(np.int32)
+        p = ctypes.c_void_p()
+        assert self.lib.s_pattern_create(ctypes.c_int32(nc), bo.ctypes, np.zeros(nc, np.int32).ctypes, rp.ctypes, ci.ctypes,
+                                         ctypes.byref(p)) == 0
+        return p
+
+    def plan(self, p, fp32):
+        q = ctypes.c_void_p()
+        return self.lib.s_plan_create(p, p, p, ctypes.c_int(fp32), ctypes.byref(q)), q
+
+    def buffers(self, p, count):
+        n, out = self.lib.s_pattern_nnz(p), []
+        for _ in range(count):
+            b = ctypes.c_void_p()
+            assert self.lib.cudaMalloc(ctypes.byref(b), ctypes.c_size_t(4 * n)) == 0
+            out.append(b)
+        return out
+
+    def launches_of(self, call):
+        """Status of a call, and how often the packed and the tile kernel and the listing ran in it."""
+        self.lib.fake_reset_launches()
+        st = call()
+        return st, [self.lib.fake_launches(k) for k in (b"mul_f32_nt_kernel", b"mul_f32_kernel", b"nt_list_kernelILb1E")]
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    from paper_2211_11681_gb300 import build
+    build.build()
+    d = tmp_path_factory.mktemp("fake")
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
+    obj, lib = str(d / "fake.o"), str(d / "libsformat_fake.so")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-fPIC", "-I", inc, "-c", os.path.join(HERE, "fake_cuda_runtime.cpp"),
+                           "-o", obj])
+    objs = [os.path.join(build.OBJ_DIR, os.path.basename(s) + ".o") for s in build.sources()]
+    subprocess.check_call(["g++", "-shared", "-Wl,-Bsymbolic", "-Wl,--no-undefined", "-o", lib] + objs + [obj, "-lgomp", "-lpthread"])
+    return Fake(lib)
+
+
+@pytest.fixture
+def calm(fake):
+    """The library with nothing made to fail, before and after a test."""
+    fake.lib.fake_pool(1 << 40)
+    yield fake
+    fake.lib.fake_fail_device(-1)
+    fake.lib.fake_fail_host(-1)
+    fake.lib.fake_pool(1 << 40)
+
+
+SIZES = [3, 20, 7, 41, 10, 1]
+
+
+@pytest.mark.parametrize("kind", ["device", "host"])
+def test_symmetric_flag_survives_a_failed_allocation(calm, kind):
+    # whichever allocation of s_plan_set_symmetric_a fails, the plan stays usable: the next product runs
+    # on the packed kernel with everything it reads in live memory, or on the tile kernel
+    from paper_2211_11681_gb300 import sformat as sf
+    L = calm.lib
+    fail = L.fake_fail_device if kind == "device" else L.fake_fail_host
+    p = calm.pattern(SIZES)
+    A, C = calm.buffers(p, 2)
+    used0, i, packed = L.fake_used(), 0, []
+    while True:
+        st, q = calm.plan(p, sf.PREC["fp32"])
+        assert st == 0
+        fail(i)
+        st = L.s_plan_set_symmetric_a(q, 1)
+        reached = (L.fake_device_calls() if kind == "device" else L.fake_host_calls()) > i
+        fail(-1)
+        assert st in (0, sf.S_ERR_NOMEM)
+        st, n = calm.launches_of(lambda: L.s_mul_masked(q, A, A, C, None))
+        assert (st, L.fake_bad()) == (0, 0), i
+        assert n[0] + n[1] == 1
+        packed.append(n[0])
+        assert L.s_plan_destroy(q) == 0
+        assert L.fake_used() == used0 and L.fake_bad() == 0
+        if not reached:
+            break
+        i += 1
+    assert i > 3 and packed[-1] == 1  # nothing failed in the last turn
