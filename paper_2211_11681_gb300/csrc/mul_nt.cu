@@ -610,9 +610,7 @@ s_status nt_configure(MulDesc* d, bool x_trans, bool y_trans, bool y_sym) {
     nt_free_side(&d->ntx);
     nt_free_side(&d->nty);
   }
-  if (st != S_ERR_NOMEM) return st;
-  cudaGetLastError();  // the failed allocation is dealt with
-  return S_OK;
+  return st == S_ERR_NOMEM ? S_OK : st;
 }
 
 static NtPack pack_of(const NtSideDesc& s, const void* src) {

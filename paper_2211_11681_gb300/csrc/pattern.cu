@@ -17,7 +17,10 @@ s_status set_error(s_status st, const std::string& msg) {
   return st;
 }
 
+// A failed allocation harms nothing but the call that made it: its record is cleared, so that the launch
+// check of the next call does not report it again.
 s_status cuda_error(cudaError_t e, const char* what) {
+  if (e == cudaErrorMemoryAllocation) cudaGetLastError();
   return set_error(e == cudaErrorMemoryAllocation ? S_ERR_NOMEM : S_ERR_CUDA,
                    std::string(what) + ": " + cudaGetErrorString(e));
 }

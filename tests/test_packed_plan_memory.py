@@ -109,3 +109,37 @@ def test_symmetric_flag_survives_a_failed_allocation(calm, kind):
             break
         i += 1
     assert i > 3 and packed[-1] == 1  # nothing failed in the last turn
+
+
+@pytest.mark.parametrize("call", ["create", "adjoint"])
+def test_failed_allocations_of_a_plan(calm, call):
+    # every device allocation of plan creation, and of the first adjoint, in turn: S_ERR_NOMEM, or a
+    # call that ran with all it reads in live memory; nothing stays allocated behind either
+    from paper_2211_11681_gb300 import sformat as sf
+    L = calm.lib
+    p = calm.pattern(SIZES)
+    A, B, C, dA, dB = calm.buffers(p, 5)
+    used0, i, refused = L.fake_used(), 0, 0
+    while True:
+        if call == "create":
+            L.fake_fail_device(i)
+        st, q = calm.plan(p, sf.PREC["fp32"])
+        if call == "adjoint":
+            assert st == 0
+            L.fake_fail_device(i)
+            st = L.s_mul_masked_adjoint(q, C, A, B, dA, dB, None)
+        reached = L.fake_device_calls() > i
+        L.fake_fail_device(-1)
+        assert st in (0, sf.S_ERR_NOMEM), (i, st)
+        refused += st != 0
+        if q:
+            st, n = calm.launches_of(lambda: L.s_mul_masked(q, A, B, C, None))
+            assert (st, n[0] + n[1]) == (0, 1), i
+            st, n = calm.launches_of(lambda: L.s_mul_masked_adjoint(q, C, A, B, dA, dB, None))
+            assert (st, n[0] + n[1]) == (0, 2), i
+            assert L.s_plan_destroy(q) == 0
+        assert (L.fake_used(), L.fake_bad()) == (used0, 0), i
+        if not reached:
+            break
+        i += 1
+    assert 0 < refused < i
