@@ -63,9 +63,12 @@ typedef enum {
  *              copies that the plan keeps and every product rewrites (s_pattern_nnz floats each,
  *              rounded up to even block widths; one copy for both when s_plan_set_symmetric_a
  *              was set and the product is called with B = A on one pattern), and the plan keeps
- *              the list of block triples (16 bytes each, up to 4 GiB; beyond that each product
- *              lists them range by range through a 256 MiB workspace).  Where there is no
- *              memory for these the product runs on a kernel that reads the operands as stored.
+ *              the list of block triples (16 bytes each) where it is at most 4 GiB and leaves half
+ *              of the device's memory free; else each product lists them range by range through
+ *              a workspace of at most 256 MiB and 1/512 of the memory free at the time.  The
+ *              two adjoints, made on the first s_mul_masked_adjoint, keep copies and lists of their
+ *              own under the same rule.  Where there is no memory for these the product runs on
+ *              a kernel that reads the operands as stored.
  *   S_BF16X3   float in, float out; each operand split into three bfloat16 parts,
  *              the six leading cross products on the tensor cores, float accumulate.
  *   S_TF32X3   float in, float out; each operand split as hi + lo, both rounded to TF32

@@ -12,9 +12,9 @@
 // operand entry some 20 to 300 times.
 //
 // Lists: the matching lambda blocks of every block of S_C (where both operands' slices start, the
-// t extent) are written once by nt_list_kernel, one warp per block, and kept by the plan when
-// they fit kNtListMax; beyond that every product lists and multiplies range after range of
-// blocks through a workspace of kNtListWork.  Intersecting inside the product kernel cost more
+// t extent) are written once by nt_list_kernel, one warp per block, and kept by the plan while there
+// is memory to spare (kNtListMax); beyond that every product lists and multiplies range after
+// range of blocks through a workspace (kNtListWork).  Intersecting inside the product kernel cost more
 // than the products of narrow blocks: in the plane the lists of a tile are 300 entries long for
 // 60 matches.
 //
@@ -71,8 +71,13 @@ constexpr int kNtBuf = 1632;     // floats of a stage buffer: 2 x 20x20x2 or 8 x
                                  // start the 8 slots 12 banks apart (conflict-free 8-byte loads)
 constexpr int kNtSlack = 64;     // a micro-tile reads up to 5 rows' pairs beyond its operand's last
 constexpr size_t kNtSmem = sizeof(float) * (kNtWarps * 2 * kNtBuf + kNtSlack);
-constexpr int64_t kNtListMax = (int64_t)4 << 30;    // bytes of lists a plan keeps
-constexpr int64_t kNtListWork = (int64_t)256 << 20; // bytes of the workspace beyond that
+// Bytes of lists a plan keeps, and of the workspace beyond that.  Lists are many times the size of a
+// matrix of narrow blocks (2.8 GB beside 87 MB at N = 6000 in space), so they are kept only while
+// they leave half of the device's memory free, and the workspace is at most 1/512 of what is
+// free: 256 plans of a batch (611 GB of lists) stay together on one GPU.
+constexpr int64_t kNtListMax = (int64_t)4 << 30;
+constexpr int64_t kNtListWork = (int64_t)256 << 20;
+constexpr int64_t kNtListLeast = (int64_t)1 << 20;
 
 // Padded t extent of a slice over nl values of t.
 __host__ __device__ __forceinline__ int nt_even(int nl) { return (nl + 1) & ~1; }
@@ -516,35 +521,47 @@ static s_status nt_build_lists(MulDesc* d) {
     }
     for (int64_t k = 0; k < nb; ++k) eptr[k + 1] = eptr[k] + h[k];
   }
-  const int64_t most = kNtListMax / (int64_t)sizeof(NtEntry), work = kNtListWork / (int64_t)sizeof(NtEntry);
-  int64_t room = 0;  // entries to allocate
-  NtRange r{0, 0, 0, 0, 0};
   for (int64_t k = 0; k < nb; ++k) {
     const int64_t ni = C->bsize[C->brow[k]], nj = C->bsize[C->colidx[k]];
     tptr[k + 1] = tptr[k] + ((ni + kTile - 1) / kTile) * ((nj + kTile - 1) / kTile);
-    // a launch counts its tiles in 32 bits
-    if (r.k1 > r.k0 && ((eptr[nb] > most && eptr[k + 1] - eptr[r.k0] > work) || tptr[k + 1] - r.t0 > INT32_MAX)) {
-      d->nt_ranges.push_back(r);
-      r = NtRange{k, k, tptr[k], tptr[k], 0};
-    }
-    r.k1 = k + 1;
-    r.t1 = tptr[k + 1];
-    room = std::max(room, eptr[r.k1] - eptr[r.k0]);
   }
-  if (nb > 0) d->nt_ranges.push_back(r);
-  for (NtRange& q : d->nt_ranges) q.base = eptr[q.k0];
   SF_CUDA(cudaMalloc(&d->nt_eptr, sizeof(int64_t) * (nb + 1)));
   SF_CUDA(cudaMemcpy(d->nt_eptr, eptr.data(), sizeof(int64_t) * (nb + 1), cudaMemcpyHostToDevice));
-  Temp dtptr;
-  SF_CUDA(cudaMalloc(&dtptr.p, sizeof(int64_t) * (nb + 1)));
-  SF_CUDA(cudaMemcpy(dtptr.p, tptr.data(), sizeof(int64_t) * (nb + 1), cudaMemcpyHostToDevice));
   SF_CUDA(cudaMalloc(&d->nt_tiles, sizeof(NtTile) * std::max<int64_t>(tptr[nb], 1)));
   if (nb > 0) {
+    Temp first;
+    SF_CUDA(cudaMalloc(&first.p, sizeof(int64_t) * (nb + 1)));
+    SF_CUDA(cudaMemcpy(first.p, tptr.data(), sizeof(int64_t) * (nb + 1), cudaMemcpyHostToDevice));
     nt_tile_kernel<<<(unsigned)((nb + 255) / 256), 256>>>(nb, C->d.bsize, C->d.brow, C->d.colidx, C->d.voff,
-                                                          (const int64_t*)dtptr.p, d->nt_eptr, d->nt_tiles);
+                                                          (const int64_t*)first.p, d->nt_eptr, d->nt_tiles);
     SF_CUDA(cudaGetLastError());
   }
-  SF_CUDA(cudaMalloc(&d->nt_ent, sizeof(NtEntry) * std::max<int64_t>(room, 1)));
+  size_t avail = 0, all = 0;
+  SF_CUDA(cudaMemGetInfo(&avail, &all));
+  const int64_t total = eptr[nb], bytes = total * (int64_t)sizeof(NtEntry);
+  const int64_t work = std::max(kNtListLeast, std::min(kNtListWork, (int64_t)(avail / 512))) / (int64_t)sizeof(NtEntry);
+  int64_t most = bytes <= kNtListMax && (int64_t)avail - bytes >= (int64_t)(all / 2) ? total : work;  // entries of a range
+  for (;; most = work) {
+    int64_t room = 0;  // entries to allocate
+    NtRange r{0, 0, 0, 0, 0};
+    d->nt_ranges.clear();
+    for (int64_t k = 0; k < nb; ++k) {
+      // (a launch counts its tiles in 32 bits)
+      if (r.k1 > r.k0 && (eptr[k + 1] - r.base > most || tptr[k + 1] - r.t0 > INT32_MAX)) {
+        d->nt_ranges.push_back(r);
+        r = NtRange{k, k, tptr[k], tptr[k], eptr[k]};
+      }
+      r.k1 = k + 1;
+      r.t1 = tptr[k + 1];
+      room = std::max(room, eptr[r.k1] - r.base);
+    }
+    if (nb > 0) d->nt_ranges.push_back(r);
+    const cudaError_t e = cudaMalloc(&d->nt_ent, sizeof(NtEntry) * std::max<int64_t>(room, 1));
+    if (e == cudaSuccess) break;
+    d->nt_ent = nullptr;
+    if (e != cudaErrorMemoryAllocation || most <= work) return cuda_error(e, "packed float product: lists");
+    cudaGetLastError();  // room for all of them at once is not to be had: range by range
+  }
   if (d->nt_ranges.size() == 1) {
     nt_list_kernel<true><<<grid, 256>>>(list_side(d->ntx), list_side(d->nty), C->d.bsize, C->d.brow, C->d.colidx, 0, nb,
                                         nullptr, d->nt_eptr, 0, d->nt_ent);

@@ -143,3 +143,71 @@ def test_failed_allocations_of_a_plan(calm, call):
             break
         i += 1
     assert 0 < refused < i
+
+
+def footprint(fake, p):
+    """Device bytes a float plan on p takes when it lists in one piece, and the lists' share."""
+    from paper_2211_11681_gb300 import sformat as sf
+    L = fake.lib
+    used = L.fake_used()
+    st, q = fake.plan(p, sf.PREC["fp32"])
+    assert st == 0
+    all_bytes = L.fake_used() - used
+    assert L.s_plan_destroy(q) == 0
+    return all_bytes
+
+
+def test_lists_leave_room(calm):
+    # 120 one-wide clusters, every block present: 1.73e6 triples, 27.6 MB of lists beside a matrix of 58 KB
+    from paper_2211_11681_gb300 import sformat as sf
+    L, lists = calm.lib, 16 * 120 ** 3
+    p = calm.pattern([1] * 120)
+    A, C = calm.buffers(p, 2)
+    rest = footprint(calm, p) - lists  # packed copies, tiles
+    assert 0 < rest < 3 << 20
+    used0 = L.fake_used()
+    # (pool, ranges of a product): kept while half of the pool stays free, else range by range in 1 MiB
+    # (1/512 of what is free is less) of 16-byte entries, rows of 120 entries a block
+    per_range = ((1 << 20) // 16) // 120 * 120
+    many = -(-120 ** 3 // per_range)
+    for pool, want in [(1 << 30, 0), (2 * (used0 + rest + lists) + 4096, 0), (2 * (used0 + rest + lists) - 65536, many),
+                       (used0 + rest + (2 << 20), many)]:
+        L.fake_pool(pool)
+        st, q = calm.plan(p, sf.PREC["fp32"])
+        assert st == 0, pool
+        if want:
+            assert L.fake_used() - used0 <= rest + (1 << 20) + 4096
+        st, n = calm.launches_of(lambda: L.s_mul_masked(q, A, A, C, None))
+        assert (st, n, L.fake_bad()) == (0, [max(want, 1), 0, want], 0), pool
+        assert L.s_plan_destroy(q) == 0 and L.fake_used() == used0
+    # not even a workspace: the tile kernel, and no packed copies kept for nothing
+    L.fake_pool(used0 + rest + (1 << 19))
+    st, q = calm.plan(p, sf.PREC["fp32"])
+    assert st == 0
+    assert L.fake_used() - used0 < rest // 2
+    st, n = calm.launches_of(lambda: L.s_mul_masked(q, A, A, C, None))
+    assert (st, n, L.fake_bad()) == (0, [0, 1, 0], 0)
+    assert L.s_plan_destroy(q) == 0
+
+
+def test_many_plans_share_a_pool(calm):
+    # as many plans as fit without lists (and a workspace of 1 MiB each) can be held together, all on
+    # the packed kernel, whatever their lists would take (32 times the pool)
+    from paper_2211_11681_gb300 import sformat as sf
+    L = calm.lib
+    p = calm.pattern([1] * 120)
+    A, C = calm.buffers(p, 2)
+    count = 64
+    pool = 256 << 20
+    assert count * 16 * 120 ** 3 > 6 * pool
+    L.fake_pool(pool)
+    plans = []
+    for _ in range(count):
+        st, q = calm.plan(p, sf.PREC["fp32"])
+        assert st == 0, len(plans)
+        assert L.s_plan_set_symmetric_a(q, 1) == 0
+        plans.append(q)
+    for q in plans:
+        st, n = calm.launches_of(lambda: L.s_mul_masked(q, A, A, C, None))
+        assert (st, n[0] > 0, n[1], L.fake_bad()) == (0, True, 0, 0)
+        assert L.s_plan_destroy(q) == 0
