@@ -70,6 +70,7 @@ constexpr int kNtKC = 20;        // largest t extent of a listed piece
 constexpr int kNtBuf = 1632;     // floats of a stage buffer: 2 x 20x20x2 or 8 x 10x10x2 slices, and room to
                                  // start the 8 slots 12 banks apart (conflict-free 8-byte loads)
 constexpr int kNtSlack = 64;     // a micro-tile reads up to 5 rows' pairs beyond its operand's last
+constexpr int kNtAhead = 6;      // tiles per resident warp from which warps take tiles ahead (see the kernel)
 constexpr size_t kNtSmem = sizeof(float) * (kNtWarps * 2 * kNtBuf + kNtSlack);
 // Bytes of lists a plan keeps, and of the workspace beyond that.  Lists are many times the size of a
 // matrix of narrow blocks (2.8 GB beside 87 MB at N = 6000 in space), so they are kept only while
@@ -347,25 +348,40 @@ __device__ __forceinline__ void nt_tile(const NtArgs& a, const NtTile& tile, flo
 // Micro-tile class of a tile edge: 0, 1 = 2 x (3, 5), 2 .. 4 = 4 x (3, 4, 5).
 __device__ __forceinline__ int nt_class(int t) { return t <= 6 ? 0 : t <= 10 ? 1 : (t - 1) >> 2; }
 
+// AHEAD: during a tile the warp already holds the next one's description and the number of the one
+// after it, which hides both fetches.  With few tiles a warp in a heavy tile would hold two that idle
+// warps could do, so below kNtAhead tiles a resident warp tiles are taken one at a time: space,
+// 20-wide, N = 500 / 1100 / 2250 55 -> 43, 134 -> 114, 446 -> 409 us; from 12 tiles a warp on
+// taking ahead is faster (plane, 10-wide, N = 2250 152 -> 145 us, N = 4000 294 -> 284 us).
+template <bool AHEAD>
 __global__ void __launch_bounds__(kNtWarps * 32, 4) mul_f32_nt_kernel(NtArgs a) {
   extern __shared__ __align__(128) float nsm[];  // [warp][buffer][kNtBuf]
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float* wbase = nsm + (size_t)w * 2 * kNtBuf;  // the warp's two stage buffers
   const uint32_t wsmem = (uint32_t)__cvta_generic_to_shared(wbase);
   wait_for_previous();
-  // the next tile is described, and the number of the one after it fetched, during the current one
-  unsigned int t = 0;
-  if (lane == 0) t = atomicAdd(a.counter, 1u);
-  t = __shfl_sync(0xffffffffu, t, 0);
+  unsigned int t = 0, tn = 0;
   NtTile nxt = {};
-  if (t < a.ntiles) nxt = a.tiles[t];
-  unsigned int tn = 0;
-  if (lane == 0) tn = atomicAdd(a.counter, 1u);
-  while (t < a.ntiles) {
-    const NtTile tile = nxt;
-    t = __shfl_sync(0xffffffffu, tn, 0);
+  if (AHEAD) {
+    if (lane == 0) t = atomicAdd(a.counter, 1u);
+    t = __shfl_sync(0xffffffffu, t, 0);
     if (t < a.ntiles) nxt = a.tiles[t];
     if (lane == 0) tn = atomicAdd(a.counter, 1u);
+  }
+  for (;;) {
+    NtTile tile;
+    if (AHEAD) {
+      if (t >= a.ntiles) break;
+      tile = nxt;
+      t = __shfl_sync(0xffffffffu, tn, 0);
+      if (t < a.ntiles) nxt = a.tiles[t];
+      if (lane == 0) tn = atomicAdd(a.counter, 1u);
+    } else {
+      if (lane == 0) t = atomicAdd(a.counter, 1u);
+      t = __shfl_sync(0xffffffffu, t, 0);
+      if (t >= a.ntiles) break;
+      tile = a.tiles[t];
+    }
     const int rc = nt_class(tile.th), cc = nt_class(tile.tw);
 #define SF_NT_CASE(R, GR, MR, Cc, GC, MC) \
   case R * 5 + Cc: nt_tile<GR, MR, GC, MC>(a, tile, wbase, wsmem, lane); break;
@@ -494,8 +510,9 @@ void nt_free_lists(MulDesc* d) {
 // workspace together (one range: the plan keeps the lists, which are written here) and
 // allocates.  All work is on the default stream and finished on return.
 static s_status nt_build_lists(MulDesc* d) {
-  SF_CUDA(cudaFuncSetAttribute(mul_f32_nt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNtSmem));
-  SF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d->nt_per_sm, mul_f32_nt_kernel, kNtWarps * 32, kNtSmem));
+  for (auto kern : {mul_f32_nt_kernel<false>, mul_f32_nt_kernel<true>})
+    SF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNtSmem));
+  SF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d->nt_per_sm, mul_f32_nt_kernel<true>, kNtWarps * 32, kNtSmem));
   d->nt_per_sm = std::max(d->nt_per_sm, 1);
   // the entries count operand offsets in 4 floats with 32 bits, t in 16
   if ((d->ntx.len >> 2) > (int64_t)UINT32_MAX || (d->nty.len >> 2) > (int64_t)UINT32_MAX) return S_OK;
@@ -669,7 +686,9 @@ s_status launch_nt(const MulDesc& d, const void* X, const void* Y, void* C, cuda
     if (r.k0 > 0) SF_CUDA(cudaMemsetAsync(d.counter, 0, sizeof(unsigned int), st));
     const int64_t want = (r.t1 - r.t0 + kNtWarps - 1) / kNtWarps;
     const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count() * d.nt_per_sm);
-    if (grid > 0) SF_CUDA(launch_overlapped(mul_f32_nt_kernel, dim3((unsigned)grid), kNtWarps * 32, kNtSmem, 0, st, a));
+    const bool ahead = r.t1 - r.t0 >= (int64_t)kNtAhead * sm_count() * d.nt_per_sm * kNtWarps;
+    auto kern = ahead ? mul_f32_nt_kernel<true> : mul_f32_nt_kernel<false>;
+    if (grid > 0) SF_CUDA(launch_overlapped(kern, dim3((unsigned)grid), kNtWarps * 32, kNtSmem, 0, st, a));
     SF_CUDA(cudaGetLastError());
   }
   return S_OK;

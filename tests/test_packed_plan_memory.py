@@ -1,5 +1,5 @@
-"""Host logic of the packed float product's plan (mul_nt.cu) when memory runs out: the library's
-object files linked with a CUDA runtime over host memory (fake_cuda_runtime.cpp), in which any
+"""Host logic of the packed float product (mul_nt.cu): what its plan does when memory runs out, and which
+kernel a product takes.  The library's object files are linked with a CUDA runtime over host memory (fake_cuda_runtime.cpp), in which any
 device or host allocation can be made to fail.  No GPU: the launches are only counted and their
 operands checked against the live allocations."""
 import ctypes
@@ -211,3 +211,18 @@ def test_many_plans_share_a_pool(calm):
         st, n = calm.launches_of(lambda: L.s_mul_masked(q, A, A, C, None))
         assert (st, n[0] > 0, n[1], L.fake_bad()) == (0, True, 0, 0)
         assert L.s_plan_destroy(q) == 0
+
+
+@pytest.mark.parametrize("nc, ahead", [(3, False), (120, False), (121, True), (160, True)])
+def test_tiles_taken_ahead(calm, nc, ahead):
+    # nc^2 tiles; the runtime has 152 SMs and 4 resident CTAs of 4 warps: the line is at 6 x 2432 = 14592
+    from paper_2211_11681_gb300 import sformat as sf
+    L = calm.lib
+    p = calm.pattern([2] * nc)
+    A, C = calm.buffers(p, 2)
+    st, q = calm.plan(p, sf.PREC["fp32"])
+    assert st == 0
+    L.fake_reset_launches()
+    assert L.s_mul_masked(q, A, A, C, None) == 0
+    assert [L.fake_launches(b"mul_f32_nt_kernelILb%d" % v) for v in (0, 1)] == [not ahead, ahead]
+    assert L.s_plan_destroy(q) == 0
