@@ -412,10 +412,11 @@ struct NtPack {
 
 // Blocks w0, w0 + nw, .. of an operand: block b (rows x cols, row-major in `src` at voff[b]), or its
 // transpose (trans), is written at poff[b] as panels of at most 20 rows, [t / 2][row][t % 2] each,
-// zeros for the padded t and up to the next multiple of 4 floats.  kNtPackLanes lanes per block
-// (a chain of dependent loads leads to each block: 8 lanes keep 4 blocks of a warp in flight); a lane
-// writes one pair of t (8 bytes) at a time.
+// zeros for the padded t and up to the next multiple of 4 floats.  LANES lanes per block; a lane writes
+// one pair of t (8 bytes) at a time.  A chain of dependent loads leads to each block: where there are
+// many, kNtPackLanes lanes keep 4 blocks of a warp in flight.
 constexpr int kNtPackLanes = 8;
+template <int LANES>
 __device__ __forceinline__ void nt_pack(const NtPack& p, int64_t w0, int64_t nw, int lane) {
   for (int64_t b = w0; b < p.nb; b += nw) {
     const int rows = p.bsize[p.brow[b]], cols = p.bsize[p.bcol[b]];
@@ -428,7 +429,7 @@ __device__ __forceinline__ void nt_pack(const NtPack& p, int64_t w0, int64_t nw,
       const int th = min(kTile, R - r0);
       const float rth = 1.0f / (float)th;
 #pragma unroll 4
-      for (int e = lane; e < th * kp; e += kNtPackLanes) {
+      for (int e = lane; e < th * kp; e += LANES) {
         const int tp = e < (1 << 20) ? __float2int_rz(((float)e + 0.5f) * rth) : e / th, r = r0 + e - tp * th;
         const float* v = s + (int64_t)r * rs + (int64_t)(2 * tp) * ts;
         d[(int64_t)r0 * kp + e] = make_float2(v[0], 2 * tp + 1 < K ? v[ts] : 0.0f);
@@ -440,15 +441,18 @@ __device__ __forceinline__ void nt_pack(const NtPack& p, int64_t w0, int64_t nw,
 
 // Packed copies of both operands (y.nb = 0: one copy serves both sides), and zero in the product's
 // tile counter.  Small products are bound by their launches, so the product's launch overlaps this
-// one's (N = 1000 in the plane 83.2 -> 80.8 us).
+// one's (N = 1000 in the plane 83.2 -> 80.8 us), and where every block of an operand can have a
+// warp at once it gets one, the second operand beside the first (grid row 1): 8 lanes a block took
+// both operands in turn, 10 us each for 20-wide blocks (N = 500 in space, two operands 75 -> 53 us).
+template <int LANES>
 __global__ void nt_prepare_kernel(NtPack x, NtPack y, unsigned int* counter) {
-  const int lane = threadIdx.x % kNtPackLanes;
-  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kNtPackLanes;
-  const int64_t nw = (int64_t)gridDim.x * blockDim.x / kNtPackLanes;
+  const int lane = threadIdx.x % LANES;
+  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LANES;
+  const int64_t nw = (int64_t)gridDim.x * blockDim.x / LANES;
   let_next_start();  // the product's CTAs take their places and wait
-  if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0u;
-  nt_pack(x, w, nw, lane);
-  nt_pack(y, w, nw, lane);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *counter = 0u;
+  if (blockIdx.y == 0) nt_pack<LANES>(x, w, nw, lane);
+  if (blockIdx.y + 1 == gridDim.y) nt_pack<LANES>(y, w, nw, lane);
 }
 
 }  // namespace
@@ -664,9 +668,13 @@ s_status launch_nt(const MulDesc& d, const void* X, const void* Y, void* C, cuda
   if (s) return s;
   const NtPack px = pack_of(d.ntx, X);
   const NtPack py = d.nty.from_x ? NtPack{} : pack_of(d.nty, Y);
-  const int64_t ctas = (std::max(px.nb, py.nb) * kNtPackLanes + 255) / 256;
-  nt_prepare_kernel<<<(int)std::max<int64_t>(1, std::min<int64_t>(ctas, (int64_t)sm_count() * 16)), 256, 0, st>>>(
-      px, py, d.counter);
+  const int64_t nb = std::max(px.nb, py.nb), ctas = (int64_t)sm_count() * 16;  // 8 CTAs an SM are resident
+  if (nb <= ctas * 8)
+    nt_prepare_kernel<32><<<dim3((unsigned)std::max<int64_t>(1, (nb + 7) / 8), py.nb > 0 ? 2 : 1), 256, 0, st>>>(
+        px, py, d.counter);
+  else
+    nt_prepare_kernel<kNtPackLanes><<<(unsigned)std::min((nb * kNtPackLanes + 255) / 256, ctas), 256, 0, st>>>(px, py,
+                                                                                                             d.counter);
   const DevPattern& pc = d.pc->d;
   for (const NtRange& r : d.nt_ranges) {
     if (d.nt_ranges.size() > 1) {

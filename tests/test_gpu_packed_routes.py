@@ -115,3 +115,17 @@ def test_range_by_range():
     again.fill_(float("nan"))
     plan.mul(a, a, again)
     np.testing.assert_array_equal(host(again), host(out))
+
+
+@pytest.mark.parametrize("nc", [120, 121, 139, 140])
+def test_small_and_large_launches(nc):
+    # around the lines where tiles are taken ahead (14592 tiles on 152 SMs) and where a block has a warp
+    # of its own in the packing (19456 blocks): nc^2 blocks of 1 to 3 rows and columns
+    from paper_2211_11681_gb300 import sformat as sf
+    bsize = 1 + np.arange(nc) % 3
+    A, B = random_bcsr(bsize, 1.0, nc), random_bcsr(bsize, 1.0, nc + 1)
+    P = pattern_of(A)
+    plan = sf.Plan(P, P, P, "fp32")
+    out = dev(np.full(len(A.val), np.nan), "float32")
+    plan.mul(dev(A.val, "float32"), dev(B.val, "float32"), out)
+    assert rel_frob(host(out), oprod.mul_masked(A, B, A, nthreads=8).val) <= 1e-5

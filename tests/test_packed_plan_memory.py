@@ -226,3 +226,18 @@ def test_tiles_taken_ahead(calm, nc, ahead):
     assert L.s_mul_masked(q, A, A, C, None) == 0
     assert [L.fake_launches(b"mul_f32_nt_kernelILb%d" % v) for v in (0, 1)] == [not ahead, ahead]
     assert L.s_plan_destroy(q) == 0
+
+
+@pytest.mark.parametrize("nc, lanes", [(3, 32), (139, 32), (140, 8)])
+def test_packing_lanes(calm, nc, lanes):
+    # a warp a block while all are resident: 152 SMs of 8 CTAs of 8 warps, twice over: 19456 blocks
+    from paper_2211_11681_gb300 import sformat as sf
+    L = calm.lib
+    p = calm.pattern([2] * nc)
+    A, B, C = calm.buffers(p, 3)
+    st, q = calm.plan(p, sf.PREC["fp32"])
+    assert st == 0
+    L.fake_reset_launches()
+    assert L.s_mul_masked(q, A, B, C, None) == 0
+    assert [L.fake_launches(b"nt_prepare_kernelILi%d" % v) for v in (8, 32)] == [lanes == 8, lanes == 32]
+    assert (L.s_plan_destroy(q), L.fake_bad()) == (0, 0)
