@@ -65,7 +65,9 @@ s_status run_add(const s_pattern_t* p, s_prec prec, double alpha, const void* A,
 // shared memory), are added in a fixed order.  What bounds it: for several vectors the FP64 pipe
 // (2 nnz nvec operations, nearly all lanes at work), for one vector the loads; the root's row,
 // which meets every cluster, is why long rows are shared (from 256 blocks on: from 64 or 128 the
-// clusters' fixed cost took 1.2 to 1.8 times as long).  Measured, N = 60000 in the plane, 10
+// clusters' fixed cost took 1.2 to 1.8 times as long; but from 32 on in a matrix of at most two rows
+// per SM, where a row's one CTA is a long chain on an idle GPU: space, 20-wide, N = 1000, one vector
+// 47 -> 18 us, 16 vectors 328 -> 131 us, the same from 16 on).  Measured, N = 60000 in the plane, 10
 // vectors (before: one thread per row and vector, A read once per vector): 21.4 -> 1.30 ms, one
 // vector 2.14 -> 0.26 ms; five pairs a lane took 1.60 ms, staging blocks and vectors in shared
 // memory as the double product does 1.33 ms and for one vector 0.47 ms.

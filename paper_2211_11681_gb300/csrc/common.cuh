@@ -42,10 +42,12 @@ struct DevPattern {
   int32_t* cscblk = nullptr;  // nblocks: CSR block index of each CSC entry
   int32_t* diag = nullptr;    // nc: block index of (nu,nu) or -1
   int32_t* roworder = nullptr;  // nc: block rows by falling number of blocks
-  int32_t nlong = 0;            // the first nlong of them have more than kLongRow blocks
+  int32_t nlong = 0;            // the first nlong of them are long (kLongRow)
 };
 
-constexpr int kLongRow = 256;  // blocks of a row beyond which a cluster of CTAs shares it (add.cu)
+// Blocks of a row beyond which a cluster of CTAs shares it (add.cu); fewer where the matrix has at most
+// two rows per SM, which would leave most of the GPU idle.
+constexpr int kLongRow = 256, kLongRowSmall = 32;
 
 }  // namespace sf
 

@@ -160,7 +160,8 @@ extern "C" s_status s_pattern_create(int32_t nc, const int64_t* block_offset, co
   std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
     return rowptr[x + 1] - rowptr[x] > rowptr[y + 1] - rowptr[y];
   });
-  while (d.nlong < nc && rowptr[order[d.nlong] + 1] - rowptr[order[d.nlong]] > kLongRow) ++d.nlong;
+  const int long_row = nc <= 2 * sm_count() ? kLongRowSmall : kLongRow;
+  while (d.nlong < nc && rowptr[order[d.nlong] + 1] - rowptr[order[d.nlong]] > long_row) ++d.nlong;
   s_status st;
   if ((st = upload(&d.roworder, order.data(), nc)) || (st = upload(&d.bsize, p->bsize.data(), nc)) || (st = upload(&d.boff, block_offset, nc + 1)) ||
       (st = upload(&d.rowptr, rowptr, nc + 1)) || (st = upload(&d.colidx, colidx, nb)) ||
