@@ -130,8 +130,8 @@ s_status s_plan_stats(s_plan plan, int64_t* triples, double* flops);
  * root-mean-square edge of at most 12 starts with 10, the others with 20.)
  * Each variant runs one timed warm-up launch; one more than twice as slow as the best so far
  * stops there, the others are timed over three more launches.  Float plans whose packed kernel
- * can run the call keep it (one product, nothing else is timed); for the others, tile and
- * row-panel shapes narrower than the root-mean-square block edge of S_C are skipped.  C is
+ * can run the call and takes more than 20 us keep it (nothing else is timed); for the others,
+ * tile and row-panel shapes narrower than the root-mean-square block edge of S_C are skipped.  C is
  * overwritten.  *chosen (optional) receives the variant index.  S_BF16X3 and S_TF32X3
  * plans have one shape (no-op).  Synchronises the stream. */
 s_status s_plan_autotune(s_plan plan, const void* A, const void* B, void* C, void* stream, int* chosen);

@@ -169,7 +169,9 @@ extern "C" s_status s_funm(s_pattern p, s_fn fn, const double* A, double* F, con
       SF_CUDA(cudaMalloc(&bA.p, w * nnz + 16));
       convert_kernel<double, float><<<g, 256, 0, st>>>(nnz, A, (float*)bA.p, 1.0);
       Ain = bA.p;
-      if (prec == S_FP32 && (s = s_plan_autotune(plan, Ain, Ain, P, st, nullptr))) return s;  // kernel shape
+      // kernel shape, unless the packed kernel runs (trying others takes longer than they can save)
+      if (prec == S_FP32 && !nt_usable(plan->fwd, Ain, Ain) && (s = s_plan_autotune(plan, Ain, Ain, P, st, nullptr)))
+        return s;
     }
     if (prec == S_FP64_DF) {
       if ((s = s_plan_autotune(plan, A, A, P, st, nullptr))) return s;  // kernel shape

@@ -1808,6 +1808,12 @@ extern "C" s_status s_mul_masked_adjoint(s_plan p, const void* dC, const void* A
   return S_OK;
 }
 
+// The autotuner stops at the packed kernel where that takes longer than this (ms).  From 200 points on the
+// tile and panel shapes took 1.1 to 15 times as long on every pattern measured (blocks 2 to 20 wide,
+// up to N = 65536); below 100 points, where a product is two launches, the 16 x 16 shape can be ahead
+// (N = 60 in space 11.0 against 14.7 us).
+constexpr float kTuneBelow = 0.02f;
+
 extern "C" s_status s_plan_autotune(s_plan p, const void* A, const void* B, void* C, void* stream, int* chosen) {
   if (!p || !A || !B || !C) return set_error(S_ERR_ARG, "s_plan_autotune: NULL argument");
   if (p->prec != S_FP32 && p->prec != S_FP64_DF && p->prec != S_FP64) {
@@ -1821,7 +1827,7 @@ extern "C" s_status s_plan_autotune(s_plan p, const void* A, const void* B, void
   cudaEvent_t e0, e1;
   SF_CUDA(cudaEventCreate(&e0));
   SF_CUDA(cudaEventCreate(&e1));
-  float best = 1e30f;
+  float best = 1e30f, packed_ms = 0.0f;
   int bestv = 0;
   s_status s = S_OK;
   // Row panels pay off only when most blocks of S_C are at most one tile wide: skip them
@@ -1835,10 +1841,9 @@ extern "C" s_status s_plan_autotune(s_plan p, const void* A, const void* B, void
     // tile shapes narrower than 20 only where the blocks are no wider than their tiles
     if (fl && !panel && !kF32Variants[v].nt && kF32Variants[v].tt < 20 && rms_edge > kF32Variants[v].tt) continue;
     if (f64 && kF64Edges[v] < 20 && rms_edge > 12.0) continue;
-    // Where the packed kernel can run nothing else is timed: on every pattern measured (blocks 1 to
-    // 40 wide, N = 1000 to 2^20) the tile and panel shapes took 1.6 to 4 times as long, and timing
-    // them took as long as 30 products.
-    if (fl && v > 0 && nt_usable(p->fwd, A, B)) break;
+    const bool packed = fl && kF32Variants[v].nt && nt_usable(p->fwd, A, B);
+    if (packed && v > 0) continue;  // the same kernel again
+    if (fl && packed_ms > kTuneBelow) break;
     if ((s = build_tiles(&p->fwd, edge_of(v)))) break;
     if (panel && (s = build_panels(&p->fwd, kF32Variants[v].tt, kF32Variants[v].panel))) break;
     p->fwd.variant = v;
@@ -1853,11 +1858,7 @@ extern "C" s_status s_plan_autotune(s_plan p, const void* A, const void* B, void
     }
     float ms = 0.0f;
     cudaEventElapsedTime(&ms, e0, e1);
-    if (fl && nt_usable(p->fwd, A, B)) {  // the only candidate
-      p->tune_ms[v] = ms;
-      bestv = v;
-      continue;
-    }
+    if (packed && ms > 50.0f * kTuneBelow) break;  // far beyond, even for a first launch: kept untimed
     if (ms > 2.0f * best / 3.0f) {
       p->tune_ms[v] = ms;
       continue;
@@ -1872,6 +1873,7 @@ extern "C" s_status s_plan_autotune(s_plan p, const void* A, const void* B, void
     }
     cudaEventElapsedTime(&ms, e0, e1);
     p->tune_ms[v] = ms / 3.0f;
+    if (packed) packed_ms = ms / 3.0f;
     if (ms < best) {
       best = ms;
       bestv = v;

@@ -29,6 +29,7 @@ std::map<std::string, int64_t>& launches() {
 }
 size_t g_total = (size_t)1 << 40, g_used = 0;
 int64_t g_dev_fail = -1, g_host_fail = -1, g_dev_calls = 0, g_host_calls = 0;
+float g_event_ms = 1.0f;
 int64_t g_bad = 0;  // launches whose operands are not in live memory
 cudaError_t g_last = cudaSuccess;
 int g_own = 0;  // > 0: an allocation of this file's own
@@ -160,6 +161,7 @@ int64_t fake_bad(void) { return g_bad; }
 // The i-th device (host) allocation from now fails; -1: none.
 void fake_fail_device(int64_t i) { g_dev_fail = i, g_dev_calls = 0; }
 void fake_fail_host(int64_t i) { g_host_fail = i, g_host_calls = 0; }
+void fake_event_ms(float ms) { g_event_ms = ms; }
 int64_t fake_device_calls(void) { return g_dev_calls; }
 int64_t fake_host_calls(void) { return g_host_calls; }
 void fake_reset_launches(void) { launches().clear(); }
@@ -233,7 +235,7 @@ cudaError_t cudaEventCreate(cudaEvent_t* e) { return *e = nullptr, cudaSuccess; 
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { return *ms = 1.0f, cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { return *ms = g_event_ms, cudaSuccess; }
 
 // ---- registration and launches --------------------------------------------------------------
 void** __cudaRegisterFatBinary(void*) {

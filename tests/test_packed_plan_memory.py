@@ -241,3 +241,23 @@ def test_packing_lanes(calm, nc, lanes):
     assert L.s_mul_masked(q, A, B, C, None) == 0
     assert [L.fake_launches(b"nt_prepare_kernelILi%d" % v) for v in (8, 32)] == [lanes == 8, lanes == 32]
     assert (L.s_plan_destroy(q), L.fake_bad()) == (0, 0)
+
+
+@pytest.mark.parametrize("ms, products", [(10.0, (1, 0)), (0.5, (4, 0)), (0.03, (4, 9))])
+def test_autotuner_stops_at_the_packed_kernel(calm, ms, products):
+    # (time of a measurement, products of the packed and of the other kernels): a first launch of 10 ms ends
+    # it, so do three of 0.17 ms each; at 0.01 ms each the 9 other shapes are tried (equal times: one
+    # launch each, the packed kernel is kept)
+    from paper_2211_11681_gb300 import sformat as sf
+    L = calm.lib
+    p = calm.pattern([2] * 5)
+    A, C = calm.buffers(p, 2)
+    st, q = calm.plan(p, sf.PREC["fp32"])
+    assert st == 0
+    L.fake_event_ms(ctypes.c_float(ms))
+    chosen = ctypes.c_int(-1)
+    L.fake_reset_launches()
+    assert L.s_plan_autotune(q, A, A, C, None, ctypes.byref(chosen)) == 0
+    n = [L.fake_launches(k) for k in (b"mul_f32_nt_kernel", b"mul_f32_kernel", b"mul_f32_panel_kernel")]
+    assert (chosen.value, n[0], n[1] + n[2]) == (0,) + products
+    assert (L.s_plan_destroy(q), L.fake_bad()) == (0, 0)
