@@ -68,8 +68,8 @@ s_status run_add(const s_pattern_t* p, s_prec prec, double alpha, const void* A,
 // clusters' fixed cost took 1.2 to 1.8 times as long; but from 32 on in a matrix of at most two rows
 // per SM, where a row's one CTA is a long chain on an idle GPU: space, 20-wide, N = 1000, one vector
 // 47 -> 18 us, 16 vectors 328 -> 131 us, the same from 16 on).  Measured, N = 60000 in the plane, 10
-// vectors (before: one thread per row and vector, A read once per vector): 21.4 -> 1.30 ms, one
-// vector 2.14 -> 0.26 ms; five pairs a lane took 1.60 ms, staging blocks and vectors in shared
+// vectors (in brackets one thread per row and vector, A read once per vector): 1.30 ms (21.4), one
+// vector 0.26 ms (2.14); five pairs a lane took 1.60 ms, staging blocks and vectors in shared
 // memory as the double product does 1.33 ms and for one vector 0.47 ms.
 constexpr int kSpWarps = 4;
 constexpr int kSpCtas = 8;     // CTAs of a cluster
@@ -199,8 +199,8 @@ __device__ __forceinline__ double cta_sum(double s, double* red) {
   return v;
 }
 
-// part[cta] = sum of a b, part[kRedCtas + cta] = sum of b b over the CTA's share.  With one CTA
-// for the whole vector (as before) a reduction over 10^7 entries took 2 ms.
+// part[cta] = sum of a b, part[kRedCtas + cta] = sum of b b over the CTA's share.  HBM-bound;
+// one CTA for the whole vector takes 2 ms for 10^7 entries.
 __global__ void __launch_bounds__(256) dot2_kernel(int64_t n, const double* __restrict__ a, const double* __restrict__ b,
                                                    double* __restrict__ part) {
   __shared__ double red[8];

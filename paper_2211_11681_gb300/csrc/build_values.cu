@@ -68,8 +68,8 @@ __device__ __forceinline__ float matern(float r, int p, float inv_ell, float sca
 // broadcast loads and a step over one input is 16 multiply-adds a lane (with the tile
 // [row][column] it was one multiply-add per two loads, one row at a time).  What bounds it: the
 // 128 bytes a clock that shared memory delivers to registers.  Every sum runs over the inputs in
-// ascending order, as before, so the values are the same to the bit.  Measured, N = 40000 on the
-// sphere (nin 16 and 20), all chunks: 79.6 -> 26.4 ms.
+// ascending order.  Measured, N = 40000 on the sphere (nin 16 and 20), all chunks: 26.4 ms (one row
+// at a time 79.6).
 __global__ void __launch_bounds__(256) eval_colfwt_kernel(Geo g, int64_t n, int64_t q0, int w,
                                                           const int32_t* __restrict__ sub,
                                                           const int32_t* __restrict__ sub_lvl_off, int nlev, int p,
@@ -166,8 +166,9 @@ __global__ void __launch_bounds__(256) eval_colfwt_kernel(Geo g, int64_t n, int6
 // columns of a cluster and holds all their inputs in registers (MAXM of them), so the outputs go
 // straight back; Q is staged once per CTA, which takes all columns of its cluster where they fit 8
 // warps, and read four outputs at a time.  HBM / L2-bound: one read
-// and one write of the rows it transforms.  Same order of the sums as before (same
-// bits); N = 40000 on the sphere, all chunks and levels: 36.8 -> 26.3 ms.
+// and one write of the rows it transforms.  Every sum runs over the inputs in
+// ascending order.  Measured, N = 40000 on the sphere, all chunks and levels: 26.3 ms (through
+// shared memory, 128 columns a CTA: 36.8).
 template <int MAXM, int VEC>
 __global__ void __launch_bounds__(256) rowfwt_reg_kernel(Geo g, const int32_t* __restrict__ lvl, int w,
                                                          float* __restrict__ U) {

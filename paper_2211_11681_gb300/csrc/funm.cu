@@ -11,7 +11,7 @@ namespace sf {
 
 // part[cta] = the CTA's share of ||T - I||_F^2 - n = sum T_ij^2 - 2 trace(T) on a pattern holding
 // every diagonal block, kRedCtas CTAs, fixed order; the host adds the shares in order.  HBM-bound
-// (one read of T); one CTA for all of it (as before) took 1.9 ms for 3.4e6 entries, this 21 us.
+// (one read of T): 21 us for 3.4e6 entries, where one CTA for all of it takes 1.9 ms.
 template <typename T>
 __global__ void __launch_bounds__(256) dist_to_identity_kernel(int64_t nnz, const T* __restrict__ v, int32_t nc,
                                                                const int32_t* __restrict__ diag,

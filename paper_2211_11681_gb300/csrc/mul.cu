@@ -110,17 +110,21 @@ __global__ void tile_fill_kernel(const int64_t* first, const int32_t* bsize, con
 // entries, 2 beyond): the S blocks' slices are staged together, and the S th tw pairs of a
 // block and an entry are dealt to the lanes, kD64Slots accumulators each, so that all 32 lanes
 // hold work whatever the block widths; the S sums of an entry are added in order at the end.
-// What bounds it: the FP64 pipe, one warp instruction every 67 clocks a scheduler whether 1 or
-// 32 lanes are active (1.0 to 1.2 TFLOP/s measured with all 32), so an instruction's empty lanes
-// are the only cost that counts: one entry per lane and lambda block filled 78 % of the lanes
-// for 10 x 10 blocks and 56 % for 6 x 6, dealing 8 blocks fills 100 %.  Staging, listing and
-// addresses run in its shadow: 16 warps an SM, one stage buffer each, while one warp waits for
-// its copies the others multiply.
-// Whole blocks are staged as the runs they are stored as.  Measured against one entry per lane
-// and lambda block: N = 4096, 6- and 10-wide blocks 7.73 -> 5.99 ms; N = 20000, 9- and 10-wide blocks
-// 25.0 -> 20.0 ms (FP64 pipe 93 % active); N = 5000 in space, 20-wide blocks 62.4 -> 62.5 ms
-// (1.17 TFLOP/s, 96 % active, at the pipe either way).
+// What bounds it: the FP64 pipe, which takes as long for 1 lane as for 32, so an instruction's empty
+// lanes and the clocks without one are the costs that count.  One entry per lane and lambda block
+// fills 78 % of the lanes for 10 x 10 blocks and 56 % for 6 x 6, dealing 8 blocks fills 100 %.
+// Staging, listing and addresses run in its shadow: 16 warps an SM, one stage buffer each, while
+// one warp waits for its copies the others multiply.  An accumulator's multiply-adds depend on one
+// another, so where a step is full and its blocks equally wide, the chains of kD64Chains
+// accumulators run side by side: one at a time the pipe idled whenever two of a scheduler's four
+// warps were staging (N = 10000 in space 244 -> 232 ms; 2 chains 244, 4 232, 5 235; in the plane N = 4096
+// 5.94 / 5.66 / 5.10 ms with 1, 4 and 3 chains; unrolling t by 2 or 4 on top 5.12 and 5.33 ms).
+// Whole blocks are staged as the runs they are stored as.  Measured (in brackets one entry per lane
+// and lambda block, 8 warps a scheduler): N = 4096, 6- and 10-wide blocks 5.10 ms (7.70); N = 20000, 9- and
+// 10-wide blocks 18.1 ms (25.0), 1.18 TFLOP/s; in space, 20-wide blocks, N = 5000 59.6 ms (62.4),
+// 1.23 TFLOP/s, N = 10000 232 ms (240).
 constexpr int kWarps = 4;
+constexpr int kD64Chains = 3;                 // slots whose chains a full step runs side by side
 constexpr int kD64Slots = 25;                 // accumulators of a lane: S th tw / 32 at most
 constexpr int kD64Buf = 1600;                 // doubles of a warp's stage buffer: S (th + tw) kc at most
 constexpr int kD64Ent = 48;                   // matching lambda blocks listed at once
@@ -129,7 +133,7 @@ constexpr size_t kD64Smem = sizeof(double) * kWarps * kD64Buf;
 struct D64Entry {
   int64_t xo, yo;  // entry offsets of op(X)'s and op(Y)'s blocks
   int32_t nl;      // lambda's width
-  uint16_t t0, kc; // first t and t extent of this piece
+  uint16_t t0, kc; // first t and t extent of this piece (blocks are at most 32767 wide)
 };
 
 template <bool TX, bool TY>
@@ -157,7 +161,8 @@ __global__ void __launch_bounds__(kWarps * 32, 4) mul_f64_kernel(MulArgs a, int 
     const int S = ne <= 100 && th + tw <= 20 ? 8 : ne <= 200 ? 4 : 2;
     const int KC = S == 2 ? 20 : 10;
     double acc[kD64Slots];
-    int off[kD64Slots];  // slot m: block s of the step, entry (r, c): s << 16 | r << 8 | c
+    // slot m: block s of the step, entry (r, c): s << 10 | r << 5 | c, two slots to a register
+    uint32_t off[(kD64Slots + 1) / 2];
     const float rne = 1.0f / (float)ne, rtw = 1.0f / (float)tw;
 #pragma unroll
     for (int m = 0; m < kD64Slots; ++m) {
@@ -165,7 +170,8 @@ __global__ void __launch_bounds__(kWarps * 32, 4) mul_f64_kernel(MulArgs a, int 
       const int i = min(lane + 32 * m, S * ne - 1);
       const int s = __float2int_rz(((float)i + 0.5f) * rne), e = i - s * ne;
       const int r = __float2int_rz(((float)e + 0.5f) * rtw);
-      off[m] = s << 16 | r << 8 | (e - r * tw);
+      const uint32_t o = (uint32_t)(s << 10 | r << 5 | (e - r * tw));
+      off[m / 2] = m & 1 ? off[m / 2] | o << 16 : o;
     }
     const int px1 = (int)a.x.ptr[nu + 1];
     int px = (int)a.x.ptr[nu];
@@ -225,21 +231,51 @@ __global__ void __launch_bounds__(kWarps * 32, 4) mul_f64_kernel(MulArgs a, int 
       }
       asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
       __syncwarp();
-      // slots of the step's blocks; a slot runs to the largest t extent of its lanes' blocks
+      // slots of the step's blocks
+      bool even = n == S;
+      for (int s = 0; s < n; ++s) even = even && (int)ent[e0 + s].kc == kc;
+      if (even) {
+        // a full step of blocks all as wide: kD64Chains slots' chains side by side
+        const int live = (S * ne + 31) >> 5;
 #pragma unroll
-      for (int m = 0; m < kD64Slots; ++m) {
-        if (32 * m >= n * ne) break;
-        const int o = off[m], s = o >> 16;
-        const int kl = s < n ? (int)ent[e0 + s].kc : 0;
-        const int ku = __reduce_max_sync(0xffffffffu, kl);
-        const int r = (o >> 8) & 255, c = o & 255;
-        const double* xp = base + s * ss + (TX ? r : r * kl);
-        const double* yp = base + s * ss + sx + (TY ? c * kl : c);
-        double v = acc[m];
+        for (int m0 = 0; m0 < kD64Slots; m0 += kD64Chains) {
+          if (m0 >= live) break;
+          const double* xp[kD64Chains];
+          const double* yp[kD64Chains];
+#pragma unroll
+          for (int v = 0; v < kD64Chains; ++v) {
+            constexpr int last = kD64Slots - 1;
+            const int m = m0 + v < last ? m0 + v : last;
+            const int o = (int)(off[m / 2] >> (16 * (m & 1))) & 0xffff, s = o >> 10, r = (o >> 5) & 31, c = o & 31;
+            xp[v] = base + s * ss + (TX ? r : r * kc);
+            yp[v] = base + s * ss + sx + (TY ? c * kc : c);
+          }
+#pragma unroll 1
+          for (int tt = 0; tt < kc; ++tt) {
+#pragma unroll
+            for (int v = 0; v < kD64Chains; ++v) {
+              if (m0 + v < kD64Slots) acc[m0 + v] = fma(*xp[v], *yp[v], acc[m0 + v]);
+              xp[v] += TX ? th : 1;
+              yp[v] += TY ? 1 : tw;
+            }
+          }
+        }
+      } else {
+        // a slot runs to the largest t extent of its lanes' blocks
+#pragma unroll
+        for (int m = 0; m < kD64Slots; ++m) {
+          if (32 * m >= n * ne) break;
+          const int o = (int)(off[m / 2] >> (16 * (m & 1))) & 0xffff, s = o >> 10, r = (o >> 5) & 31, c = o & 31;
+          const int kl = s < n ? (int)ent[e0 + s].kc : 0;
+          const int ku = __reduce_max_sync(0xffffffffu, kl);
+          const double* xp = base + s * ss + (TX ? r : r * kl);
+          const double* yp = base + s * ss + sx + (TY ? c * kl : c);
+          double v = acc[m];
 #pragma unroll 2
-        for (int tt = 0; tt < ku; ++tt, xp += TX ? th : 1, yp += TY ? 1 : tw)
-          if (tt < kl) v = fma(*xp, *yp, v);
-        acc[m] = v;
+          for (int tt = 0; tt < ku; ++tt, xp += TX ? th : 1, yp += TY ? 1 : tw)
+            if (tt < kl) v = fma(*xp, *yp, v);
+          acc[m] = v;
+        }
       }
       __syncwarp();
       e0 += n;

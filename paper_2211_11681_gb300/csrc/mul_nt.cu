@@ -40,22 +40,21 @@
 // Sums: even and odd t are two float partials per entry; after the first step, then every 4 (8 of
 // wide tiles), they are added and folded into the running sum with an error-free two-sum,
 // the rounding error carried in the partial.  The lists run from coarse to fine clusters, so
-// the first step holds the largest terms: folded at once, it no longer makes the small terms
-// that follow round at its size.  At the end the groups' sums are combined the same way in
-// group order.  The order is fixed (deterministic).  Error against 64 bits, geometric mean over 8
-// matrices of 500 to 9900 points: 0.4e-7 to 1.4e-7 in the four families with 20- and 10-wide
-// blocks (1.1e-7 to 4.0e-7 with the replaced kernel's folds every 4 lambda blocks).  Narrow tiles
-// folded only every 16 steps were 0.8 % faster, but left the float square root at N = 2000 in space,
-// whose factors are near the identity, 2.6e-7 off (1.1e-7 now, 2.0e-7 with the replaced kernel).
-// Within a block t runs downwards, so a cluster's coarsest samplets, the largest terms of the
-// dominant entries, are added last and round once (they alone decide the error's norm on matrices
-// of a few thousand points: N = 5000 in the plane 6.8e-8 -> 1.7e-8 over 6 matrices, 1.4e-7 with the
-// replaced kernel); upwards was 0.4 % faster.
+// the first step holds the largest terms: folded at once, it does not make the small terms that
+// follow round at its size.  At the end the groups' sums are combined the same way in group
+// order.  The order is fixed (deterministic).  Within a block t runs downwards, so a cluster's
+// coarsest samplets, the largest terms of the dominant entries, are added last and round once.
+// Error against 64 bits, geometric mean over 8 matrices of 500 to 9900 points: 0.2e-7 to 1.4e-7
+// in the four families with 20- and 10-wide blocks.  Folding narrow tiles only every 16 steps is
+// 0.8 % faster, but leaves the float square root at N = 2000 in space, whose factors are near the
+// identity, 2.6e-7 off instead of 1.1e-7; t upwards is 0.4 % faster and takes the error at
+// N = 5000 in the plane from 1.7e-8 to 6.8e-8.
 //
-// Measured against the kernel this replaces (K-major slices, in-kernel intersection, one half-warp
-// per lambda block): N = 50000 in the plane, 10-wide blocks, B not symmetric 9.27 -> 4.0 ms; N = 65536 in
-// space, 20-wide blocks, B = A symmetric 39.1 -> 30.5 ms (37.6 TFLOP/s); N = 1000 in the plane
-// 192 -> 83 us; three products of a gradient step, N = 6000, 10-wide blocks 107.6 -> 35.6 ms.
+// Measured (in brackets a kernel with K-major slices that intersects the lists itself, one half-warp
+// per lambda block): N = 50000 in the plane, 10-wide blocks, B not symmetric 3.98 ms (9.27); N = 65536 in
+// space, 20-wide blocks, B = A symmetric 30.5 ms, 37.5 TFLOP/s (39.1); N = 1000 in the plane 60 us
+// (192); N = 500 in space, 20-wide 43 us (45 symmetric, 56 not); three products of a gradient
+// step, N = 6000, 10-wide blocks 35.6 ms (107.6).
 #include <algorithm>
 #include <cstring>
 #include <new>
@@ -75,7 +74,11 @@ constexpr size_t kNtSmem = sizeof(float) * (kNtWarps * 2 * kNtBuf + kNtSlack);
 // Bytes of lists a plan keeps, and of the workspace beyond that.  Lists are many times the size of a
 // matrix of narrow blocks (2.8 GB beside 87 MB at N = 6000 in space), so they are kept only while
 // they leave half of the device's memory free, and the workspace is at most 1/512 of what is
-// free: 256 plans of a batch (611 GB of lists) stay together on one GPU.
+// free: 256 plans of a batch (611 GB of lists) stay together on one GPU.  Range by range a product
+// lists again and drains between ranges: N = 65536 in space, 20-wide 30.9 -> 33.7 ms, N = 250000 in the
+// plane, 10-wide 19.9 -> 32.1 ms (39.1 with 64 MiB of workspace, 29.0 with 1 GiB).  4 GiB hold the
+// lists of 2.7e8 block triples; beyond, N = 10^6 in the plane (7.9 GB) takes 139 ms, 85 with its lists
+// kept, N = 10^5 in space (11.2 GB) 321 and 271 ms.
 constexpr int64_t kNtListMax = (int64_t)4 << 30;
 constexpr int64_t kNtListWork = (int64_t)256 << 20;
 constexpr int64_t kNtListLeast = (int64_t)1 << 20;
@@ -187,7 +190,7 @@ __global__ void nt_tile_kernel(int64_t nb, const int32_t* __restrict__ bsize, co
 }
 
 // 16-byte asynchronous copy global -> shared: through L1 for the narrow tiles (GL = 4), whose
-// neighbours re-read the same small slices soon (gradient step at N = 6000 36.6 -> 34.9 ms before the folds every 4 steps), past
+// neighbours re-read the same small slices soon (gradient step at N = 6000 in space 5 % faster), past
 // L1 for the others (with it N = 65536 in space took 35.4 instead of 30.4 ms).
 template <bool L1>
 __device__ __forceinline__ void nt_cp16(uint32_t dst, const float* src) {
@@ -414,7 +417,8 @@ struct NtPack {
 // transpose (trans), is written at poff[b] as panels of at most 20 rows, [t / 2][row][t % 2] each,
 // zeros for the padded t and up to the next multiple of 4 floats.  LANES lanes per block; a lane writes
 // one pair of t (8 bytes) at a time.  A chain of dependent loads leads to each block: where there are
-// many, kNtPackLanes lanes keep 4 blocks of a warp in flight.
+// many, kNtPackLanes lanes keep 4 blocks of a warp in flight (N = 50000 in the plane 183 us, a warp to
+// a block 306).
 constexpr int kNtPackLanes = 8;
 template <int LANES>
 __device__ __forceinline__ void nt_pack(const NtPack& p, int64_t w0, int64_t nw, int lane) {
