@@ -121,8 +121,8 @@ __global__ void tile_fill_kernel(const int64_t* first, const int32_t* bsize, con
 // 5.94 / 5.66 / 5.10 ms with 1, 4 and 3 chains; unrolling t by 2 or 4 on top 5.12 and 5.33 ms).
 // Whole blocks are staged as the runs they are stored as.  Measured (in brackets one entry per lane
 // and lambda block, 8 warps a scheduler): N = 4096, 6- and 10-wide blocks 5.10 ms (7.70); N = 20000, 9- and
-// 10-wide blocks 18.1 ms (25.0), 1.18 TFLOP/s; in space, 20-wide blocks, N = 5000 59.6 ms (62.4),
-// 1.23 TFLOP/s, N = 10000 232 ms (240).
+// 10-wide blocks 18.1 ms (25.0), 1.18 TFLOP/s, FP64 pipe 97.9 % active; in space, 20-wide blocks,
+// N = 5000 59.6 ms (62.4), 1.23 TFLOP/s, 99.3 % active, N = 10000 232 ms (240).
 constexpr int kWarps = 4;
 constexpr int kD64Chains = 3;                 // slots whose chains a full step runs side by side
 constexpr int kD64Slots = 25;                 // accumulators of a lane: S th tw / 32 at most
@@ -1845,9 +1845,9 @@ extern "C" s_status s_mul_masked_adjoint(s_plan p, const void* dC, const void* A
 }
 
 // The autotuner stops at the packed kernel where that takes longer than this (ms).  From 200 points on the
-// tile and panel shapes took 1.1 to 15 times as long on every pattern measured (blocks 2 to 20 wide,
-// up to N = 65536); below 100 points, where a product is two launches, the 16 x 16 shape can be ahead
-// (N = 60 in space 11.0 against 14.7 us).
+// best of the other shapes it may try took 1.1 to 5.3 times as long on every pattern measured (blocks 2
+// to 20 wide, up to N = 65536); below 100 points, where a product is two launches, one of them can be
+// ahead (16 x 16, N = 60 in space 11.0 against 14.7 us).
 constexpr float kTuneBelow = 0.02f;
 
 extern "C" s_status s_plan_autotune(s_plan p, const void* A, const void* B, void* C, void* stream, int* chosen) {

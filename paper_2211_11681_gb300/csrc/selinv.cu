@@ -40,7 +40,7 @@
 //
 // Measured, factorization and inversion in the plane, 10-wide blocks (in brackets one entry per lane
 // and term, sums split for sixteen warps a scheduler): N = 4096 22.7 ms (37.7), N = 8192 53.9 ms
-// (82.8), N = 16384 172 ms (228), N = 65536 1.50 s (1.88), 71 % of the measured FP64 rate there.
+// (82.8), N = 16384 172 ms (228), N = 65536 1.50 s (1.88), 0.75 TFLOP/s.
 //
 // Every entry a launch reads was written by an earlier launch (descendants sit on lower
 // levels, ancestors on higher ones) or by its own CTA before a barrier, so the kernels need
