@@ -160,7 +160,7 @@ struct MulDesc {
                                      // device, so the host reads it without a sync
   bool tc_sym = false;             // symmetric plan: B = A, Y read through its stored transpose
   NtSideDesc ntx, nty;             // packed float product sides (S_FP32)
-  int64_t* nt_eptr = nullptr;      // first entry of each block of S_C (device, nblocks + 1)
+  int64_t* nt_eptr = nullptr;      // first entry, then first tile, of each block of S_C (device, twice nblocks + 1)
   NtTile* nt_tiles = nullptr;      // tiles of S_C in block order
   NtEntry* nt_ent = nullptr;       // lists of the current range (nullptr: side or lists missing)
   std::vector<NtRange> nt_ranges;  // one: the plan keeps all lists

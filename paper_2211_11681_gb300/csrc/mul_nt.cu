@@ -528,42 +528,35 @@ static s_status nt_build_lists(MulDesc* d) {
     if (q->d.max_bsize > 65000) return S_OK;
   const s_pattern_t* C = d->pc;
   const int64_t nb = C->d.nblocks;
-  std::vector<int64_t> eptr(nb + 1, 0), tptr(nb + 1, 0);
-  struct Temp {  // device memory of this call
-    void* p = nullptr;
-    ~Temp() { cudaFree(p); }
-  };
+  // where each block's list and tiles start; on the device one buffer, whose second half holds the
+  // lists' lengths first (allocations and copies are most of the time this takes for small plans)
+  std::vector<int64_t> start(2 * (nb + 1), 0);
+  int64_t *eptr = start.data(), *tptr = eptr + nb + 1;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((nb + 7) / 8, (int64_t)sm_count() * 64));
-  {
-    Temp cnt;
+  SF_CUDA(cudaMalloc(&d->nt_eptr, sizeof(int64_t) * start.size()));
+  if (nb > 0) {
     std::vector<int32_t> h(nb);
-    SF_CUDA(cudaMalloc(&cnt.p, sizeof(int32_t) * std::max<int64_t>(nb, 1)));
-    if (nb > 0) {
-      nt_list_kernel<false><<<grid, 256>>>(list_side(d->ntx), list_side(d->nty), C->d.bsize, C->d.brow, C->d.colidx, 0, nb,
-                                           (int32_t*)cnt.p, nullptr, 0, nullptr);
-      SF_CUDA(cudaGetLastError());
-      SF_CUDA(cudaMemcpy(h.data(), cnt.p, sizeof(int32_t) * nb, cudaMemcpyDeviceToHost));
+    int32_t* cnt = (int32_t*)(d->nt_eptr + nb + 1);
+    nt_list_kernel<false><<<grid, 256>>>(list_side(d->ntx), list_side(d->nty), C->d.bsize, C->d.brow, C->d.colidx, 0, nb,
+                                         cnt, nullptr, 0, nullptr);
+    SF_CUDA(cudaGetLastError());
+    SF_CUDA(cudaMemcpy(h.data(), cnt, sizeof(int32_t) * nb, cudaMemcpyDeviceToHost));
+    for (int64_t k = 0; k < nb; ++k) {
+      const int64_t ni = C->bsize[C->brow[k]], nj = C->bsize[C->colidx[k]];
+      eptr[k + 1] = eptr[k] + h[k];
+      tptr[k + 1] = tptr[k] + ((ni + kTile - 1) / kTile) * ((nj + kTile - 1) / kTile);
     }
-    for (int64_t k = 0; k < nb; ++k) eptr[k + 1] = eptr[k] + h[k];
   }
-  for (int64_t k = 0; k < nb; ++k) {
-    const int64_t ni = C->bsize[C->brow[k]], nj = C->bsize[C->colidx[k]];
-    tptr[k + 1] = tptr[k] + ((ni + kTile - 1) / kTile) * ((nj + kTile - 1) / kTile);
-  }
-  SF_CUDA(cudaMalloc(&d->nt_eptr, sizeof(int64_t) * (nb + 1)));
-  SF_CUDA(cudaMemcpy(d->nt_eptr, eptr.data(), sizeof(int64_t) * (nb + 1), cudaMemcpyHostToDevice));
+  SF_CUDA(cudaMemcpy(d->nt_eptr, start.data(), sizeof(int64_t) * start.size(), cudaMemcpyHostToDevice));
   SF_CUDA(cudaMalloc(&d->nt_tiles, sizeof(NtTile) * std::max<int64_t>(tptr[nb], 1)));
   if (nb > 0) {
-    Temp first;
-    SF_CUDA(cudaMalloc(&first.p, sizeof(int64_t) * (nb + 1)));
-    SF_CUDA(cudaMemcpy(first.p, tptr.data(), sizeof(int64_t) * (nb + 1), cudaMemcpyHostToDevice));
     nt_tile_kernel<<<(unsigned)((nb + 255) / 256), 256>>>(nb, C->d.bsize, C->d.brow, C->d.colidx, C->d.voff,
-                                                          (const int64_t*)first.p, d->nt_eptr, d->nt_tiles);
+                                                          d->nt_eptr + nb + 1, d->nt_eptr, d->nt_tiles);
     SF_CUDA(cudaGetLastError());
   }
-  size_t avail = 0, all = 0;
-  SF_CUDA(cudaMemGetInfo(&avail, &all));
   const int64_t total = eptr[nb], bytes = total * (int64_t)sizeof(NtEntry);
+  size_t avail = 0, all = 0;
+  if (bytes > kNtListLeast) SF_CUDA(cudaMemGetInfo(&avail, &all));
   const int64_t work = std::max(kNtListLeast, std::min(kNtListWork, (int64_t)(avail / 512))) / (int64_t)sizeof(NtEntry);
   int64_t most = bytes <= kNtListMax && (int64_t)avail - bytes >= (int64_t)(all / 2) ? total : work;  // entries of a range
   for (;; most = work) {
